@@ -1134,9 +1134,8 @@ struct Wolfe {
 
 // ------------------------------------------------------------------ exact QP in float32
 // The same minimum-norm-point method as Wolfe<M, R> (see there), arranged
-// for speed in float32: one QP per thread with every array in registers
-// (loops fully unrolled over the at most 7 points), the nearest point of the
-// affine hull found by a QR factorisation of the differences
+// for speed in float32: one QP per thread, the nearest point of the affine
+// hull found by a QR factorisation of the differences
 // D = [p_1 - p_0, ...] (modified Gram-Schmidt, each column orthogonalised
 // twice) instead of the normal equations D^T D, whose float32 conditioning
 // (kappa^2) cost accuracy; and vertices held as codes: per contact its best
@@ -1150,59 +1149,71 @@ struct Wolfe {
 // nearest one at float32 resolution, and its gap bound may then be loose);
 // or after max_calls oracle calls.  Returns the calls used,
 // negated when the cap stopped it; gap receives the last Frank-Wolfe gap.
-template <int M>
+// SMEM: G lies in shared memory, and every read of it is an instruction of
+// its own (lds32): left to itself the compiler keeps the 18m values that the
+// oracle reads twice in registers, 249 instead of 168.
+template <int M, bool SMEM = true>
 struct ExactQP {
   static constexpr int NV = 3 * M, K = 7;
+  static constexpr int VW = 2 * K;  // words of vertex storage per QP: K codes, K fractional forces
   struct Vtx {
     int code;    // bits 4i..4i+2: contact i's edge k; bit 4i+3: f_i = 1; bits 20..22: fractional contact (7: none)
     float frac;  // the fractional contact's f
   };
   // edge tip directions (1, mu cos(k pi/4), mu sin(k pi/4)): cos, sin of k pi/4
-  __device__ static float ck(int k) {
+  __device__ static constexpr float ck(int k) {
     const float h = 0.70710678118654752f;
     return k == 0 ? 1.f : k == 1 ? h : k == 2 ? 0.f : k == 3 ? -h : k == 4 ? -1.f : k == 5 ? -h : k == 6 ? 0.f : h;
   }
-  __device__ static float sk(int k) { return ck((k + 6) & 7); }
+  __device__ static constexpr float sk(int k) { return ck((k + 6) & 7); }
+  // cos and sin of edge k for the lookups by a lane's own k, in shared memory
+  static constexpr int EDGE_WORDS = 16;
+  __device__ static void fill_edges(float* e) {
+    for (int k = threadIdx.x; k < 8; k += blockDim.x) {
+      e[2 * k] = ck(k);
+      e[2 * k + 1] = sk(k);
+    }
+  }
   // f_i of contact i in a vertex
   __device__ static float f_of(const Vtx& v, int i) {
     if (((v.code >> 20) & 7) == i) return v.frac;
     return ((v.code >> (4 * i + 3)) & 1) ? 1.f : 0.f;
   }
+  __device__ __forceinline__ static float ld(const float* p) {
+    if constexpr (SMEM) return lds32(p);
+    else return *p;
+  }
   // linear oracle: the vertex of C minimising x . (G v) (continuous knapsack
   // over the contacts' best edges), and its point q = G v - b
-  __device__ static Vtx oracle(const float* G, const float* b, const float* x, const AdmmCfg& c, float* q) {
-    float gy[NV];
-#pragma unroll
-    for (int a = 0; a < NV; ++a) {
-      float s = 0.f;
-#pragma unroll
-      for (int r = 0; r < 6; ++r) s = fmaf(G[r * NV + a], x[r], s);
-      gy[a] = s;
-    }
+  __device__ static Vtx oracle(const float* G, const float* b, const float* x, const AdmmCfg& c, const float* edge,
+                               float* q) {
     float cb[M];
-    int kb[M];
-#pragma unroll
-    for (int i = 0; i < M; ++i) {
-      // every multiply-add spelled out: the value must not depend on the
-      // code the solve is inlined into (the compiler's contraction does)
-      float best = fmaf(c.mu, gy[3 * i + 1], gy[3 * i]);
-      int k0 = 0;
-#pragma unroll
-      for (int k = 1; k < 8; ++k) {
-        const float v = fmaf(c.mu, fmaf(ck(k), gy[3 * i + 1], __fmul_rn(sk(k), gy[3 * i + 2])), gy[3 * i]);
-        if (v < best) best = v, k0 = k;
-      }
-      cb[i] = best;
-      kb[i] = k0;
-    }
     Vtx v;
     v.code = 7 << 20;
     v.frac = 0.f;
     float sum = 0.f;
 #pragma unroll
     for (int i = 0; i < M; ++i) {
-      v.code |= kb[i] << (4 * i);
-      if (cb[i] < 0.f) {
+      float gy[3];
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        float s = 0.f;
+#pragma unroll
+        for (int r = 0; r < 6; ++r) s = fmaf(ld(G + r * NV + 3 * i + a), x[r], s);
+        gy[a] = s;
+      }
+      // every multiply-add spelled out: the value must not depend on the
+      // code the solve is inlined into (the compiler's contraction does)
+      float best = fmaf(c.mu, gy[1], gy[0]);
+      int k0 = 0;
+#pragma unroll
+      for (int k = 1; k < 8; ++k) {
+        const float val = fmaf(c.mu, fmaf(ck(k), gy[1], __fmul_rn(sk(k), gy[2])), gy[0]);
+        if (val < best) best = val, k0 = k;
+      }
+      cb[i] = best;
+      v.code |= k0 << (4 * i);
+      if (best < 0.f) {
         v.code |= 1 << (4 * i + 3);
         sum += 1.f;
       }
@@ -1228,278 +1239,328 @@ struct ExactQP {
       sum += add;
       if (add < 1.f) break;
     }
-    point(G, b, v, c, q);
+    point(G, b, v, c, edge, q);
     return v;
   }
-  __device__ static void point(const float* G, const float* b, const Vtx& v, const AdmmCfg& c, float* q) {
+  __device__ static void point(const float* G, const float* b, const Vtx& v, const AdmmCfg& c, const float* edge,
+                               float* q) {
 #pragma unroll
     for (int r = 0; r < 6; ++r) q[r] = -b[r];
 #pragma unroll
     for (int i = 0; i < M; ++i) {
       const float f = f_of(v, i);
-      if (f != 0.f) {
-        const int k = (v.code >> (4 * i)) & 7;
-        const float fm = __fmul_rn(f, c.mu), fd = __fmul_rn(fm, ck(k)), fe = __fmul_rn(fm, sk(k));
+      const float* e = edge + 2 * ((v.code >> (4 * i)) & 7);
+      const float fm = __fmul_rn(f, c.mu), fd = __fmul_rn(fm, e[0]), fe = __fmul_rn(fm, e[1]);
+      // no branch on f: the lanes of a warp push with different contacts
 #pragma unroll
-        for (int r = 0; r < 6; ++r)
-          q[r] = fmaf(f, G[r * NV + 3 * i], fmaf(fd, G[r * NV + 3 * i + 1], fmaf(fe, G[r * NV + 3 * i + 2], q[r])));
+      for (int r = 0; r < 6; ++r) {
+        const float* g = G + r * NV + 3 * i;
+        const float s = fmaf(f, ld(g), fmaf(fd, ld(g + 1), fmaf(fe, ld(g + 2), q[r])));
+        q[r] = f != 0.f ? s : q[r];
       }
     }
   }
-  __device__ static void accumulate_y(const Vtx& v, float w, const AdmmCfg& c, float* y) {
+  __device__ static void accumulate_y(const Vtx& v, float w, const AdmmCfg& c, const float* edge, float* y) {
 #pragma unroll
     for (int i = 0; i < M; ++i) {
       const float fo = f_of(v, i), f = __fmul_rn(w, fo), fm = __fmul_rn(f, c.mu);
-      const int k = (v.code >> (4 * i)) & 7;
+      const float* e = edge + 2 * ((v.code >> (4 * i)) & 7);
       y[3 * i] = fmaf(w, fo, y[3 * i]);
-      y[3 * i + 1] = fmaf(fm, ck(k), y[3 * i + 1]);
-      y[3 * i + 2] = fmaf(fm, sk(k), y[3 * i + 2]);
+      y[3 * i + 1] = fmaf(fm, e[0], y[3 * i + 1]);
+      y[3 * i + 2] = fmaf(fm, e[1], y[3 * i + 2]);
     }
   }
-  // nearest point of the affine hull of P[0..n-1]: weights al (sum 1);
-  // false when the differences are (numerically) dependent.  The loops over
-  // the working set run to n, not unrolled to K: the unrolled form missed the
-  // instruction cache in the fused step (17% slower there, the same alone)
-  __device__ static bool affine_min(const float (&P)[K][6], int n, float (&al)[K]) {
-    float U[K - 1][6], R[K - 1][K - 1], sc = 1.f;
-#pragma unroll 1
-    for (int i = 0; i < n; ++i)
-#pragma unroll
-      for (int r = 0; r < 6; ++r) sc = fmaxf(sc, fabsf(P[i][r]));
-#pragma unroll 1
-    for (int j = 0; j + 1 < n; ++j) {
-      float u[6];
-#pragma unroll
-      for (int r = 0; r < 6; ++r) u[r] = P[j + 1][r] - P[0][r];
-#pragma unroll 1
-      for (int i = 0; i < j; ++i) R[i][j] = 0.f;
-#pragma unroll
-      for (int pass = 0; pass < 2; ++pass)
-#pragma unroll 1
-        for (int i = 0; i < j; ++i) {
-          float d = 0.f;
-#pragma unroll
-          for (int r = 0; r < 6; ++r) d = fmaf(U[i][r], u[r], d);
-          R[i][j] += d;
-#pragma unroll
-          for (int r = 0; r < 6; ++r) u[r] = fmaf(-d, U[i][r], u[r]);
-        }
-      float nn = 0.f;
-#pragma unroll
-      for (int r = 0; r < 6; ++r) nn = fmaf(u[r], u[r], nn);
-      const float rjj = sqrtf(nn);
-      if (!(rjj > 1e-6f * sc)) return false;
-      R[j][j] = rjj;
-      const float inv = 1.f / rjj;
-#pragma unroll
-      for (int r = 0; r < 6; ++r) U[j][r] = u[r] * inv;
-    }
-    float a1[K - 1];
-#pragma unroll 1
-    for (int j = n - 2; j >= 0; --j) {
-      float s = 0.f;
-#pragma unroll
-      for (int r = 0; r < 6; ++r) s = fmaf(-U[j][r], P[0][r], s);
-#pragma unroll 1
-      for (int k = n - 2; k > j; --k) s = fmaf(-R[j][k], a1[k], s);
-      a1[j] = s / R[j][j];
-    }
-    float a0 = 1.f;
-#pragma unroll 1
-    for (int j = 0; j + 1 < n; ++j) {
-      al[j + 1] = a1[j];
-      a0 -= a1[j];
-    }
-    al[0] = a0;
-    return true;
+  // c ? a : b as one selp: written with ?: (or if), a chain over the points
+  // becomes an indexed load and puts the whole set in local memory
+  __device__ __forceinline__ static float pick(bool c, float a, float b) {
+    float r;
+    asm("{ .reg .pred p; setp.ne.u32 p, %3, 0; selp.f32 %0, %1, %2, p; }" : "=f"(r) : "f"(a), "f"(b), "r"((unsigned)c));
+    return r;
   }
-  // The working set ("corral"): n points with their vertex codes and weights.
-  struct Corral {
-    int n;
-    Vtx V[K];
-    float lam[K];
-  };
-  // Minor cycles of Wolfe's method on (P, C): the nearest point of the
-  // affine hull of the set; while it leaves the simplex, step towards it
-  // until a weight reaches 0 and drop that point.  Returns false when the
-  // points turned out dependent (the last one is dropped, the weights kept).
-  __device__ static bool minor(float (&P)[K][6], Corral& C) {
-    int& n = C.n;
-#pragma unroll 1
-    for (int guard = 0; guard < 2 * K; ++guard) {
-      float al[K];
-      if (!affine_min(P, n, al)) {  // dependent points: drop the last one, keep the current weights
-        --n;
-        float tot = 0.f;
-#pragma unroll
-        for (int i = 0; i < K; ++i) tot += i < n ? C.lam[i] : 0.f;
-        const float it = tot > 0.f ? 1.f / tot : 0.f;
-#pragma unroll
-        for (int i = 0; i < K; ++i) C.lam[i] = i < n ? (tot > 0.f ? C.lam[i] * it : (i == 0 ? 1.f : 0.f)) : 0.f;
-        return false;
-      }
-      bool inside = true;
-#pragma unroll
-      for (int i = 0; i < K; ++i)
-        if (i < n) inside = inside && al[i] > 0.f;
-      if (inside) {
-#pragma unroll
-        for (int i = 0; i < K; ++i) C.lam[i] = i < n ? al[i] : 0.f;
-        return true;
-      }
-      float th = 1.f;
-      int drop = -1;
-#pragma unroll
-      for (int i = 0; i < K; ++i)
-        if (i < n && al[i] <= 0.f) {
-          const float den = C.lam[i] - al[i];
-          const float ti = den > 0.f ? C.lam[i] / den : 0.f;
-          if (drop < 0 || ti < th) th = ti, drop = i;
-        }
-      float tot = 0.f;
-#pragma unroll
-      for (int i = 0; i < K; ++i)
-        if (i < n) {
-          C.lam[i] = i == drop ? 0.f : fmaxf(fmaf(th, al[i] - C.lam[i], C.lam[i]), 0.f);
-          tot += C.lam[i];
-        }
-      // compact: move the last point into the dropped slot
-      const int last = n - 1;
-#pragma unroll
-      for (int i = 0; i < K; ++i)
-        if (i == drop && drop != last) {
-#pragma unroll
-          for (int j = 0; j < K; ++j)
-            if (j == last) {
-              C.V[i] = C.V[j];
-              C.lam[i] = C.lam[j];
-#pragma unroll
-              for (int r = 0; r < 6; ++r) P[i][r] = P[j][r];
-            }
-        }
-      --n;
-      const float it = tot > 0.f ? 1.f / tot : 0.f;
-#pragma unroll
-      for (int i = 0; i < K; ++i) C.lam[i] = i < n ? C.lam[i] * it : 0.f;
-      if (n == 1) {
-        C.lam[0] = 1.f;
-        return true;
-      }
-    }
-    return true;
-  }
+  __device__ static constexpr int ri(int i, int j) { return j * (j - 1) / 2 + i; }  // R_ij, i < j, packed by columns
 
-  // Solves the QP starting from the corral C (C.n == 0: a cold start at the
-  // oracle's vertex for y = 0); C receives the final corral, which a later
-  // solve of a nearby QP (the next upper step's G) can start from: its
-  // points are recomputed for the new G and the minor cycles make it a valid
-  // corral again before the first oracle call.
-  __device__ static int solve(const float* G, const float* t, const AdmmCfg& c, int max_calls, Corral& C, float* y,
-                              float& Q, float& gap) {
+  // Solves the QP starting from the corral (n points, their vertices in
+  // vs, their weights lam; n <= 0: a cold start at the oracle's vertex for
+  // y = 0); it receives the final corral, which a later solve of a nearby QP
+  // (the next upper step's G) can start from: its points are recomputed for
+  // the new G and minor cycles make it a valid corral again before the first
+  // oracle call.  Vertex i's code is vs[i * stride], its fractional force
+  // vs[(K + i) * stride]; edge: the table of fill_edges.
+  //
+  // The method is a loop of passes.  In a pass, a QP that needs a vertex
+  // calls the oracle, and every QP takes one minor cycle: the nearest point
+  // of the affine hull of its set, and the step to it or towards it until a
+  // weight reaches 0 and that point drops out (then the next pass starts with
+  // another minor cycle).  The lanes of a warp so run the same code at the
+  // same time whatever their QPs do; with the minor cycles as a loop inside
+  // the oracle's, 8.6 of 32 lanes were active per instruction.  The QR factors
+  // stay between passes and only the columns of points that changed are
+  // formed again (one, when a vertex was added), with the same operations in
+  // the same order as a new factorisation.  All loops over the set are
+  // unrolled and masked, so that it lives in registers: indexed by a lane's
+  // own counters it went to local memory.
+  __device__ static int solve(const float* G, const float* t, const AdmmCfg& c, const float* edge, int max_calls,
+                              int& n_io, float (&lam)[K], float* vs, int stride, float* y, float& Q, float& gap) {
     float b[6];
 #pragma unroll
-    for (int r = 0; r < 6; ++r) b[r] = c.beta * t[r];
-    float P[K][6], x[6];
-    int calls = 0;
-    if (C.n <= 0 || C.n > K) {  // cold: the oracle's vertex at y = 0 (x = -b)
+    for (int r = 0; r < 6; ++r) b[r] = __fmul_rn(c.beta, t[r]);
+    float P[K][6], U[K - 1][6], R[(K - 1) * (K - 2) / 2], D[K - 1];
 #pragma unroll
-      for (int r = 0; r < 6; ++r) x[r] = -b[r];
-      C.V[0] = oracle(G, b, x, c, P[0]);
-      C.n = 1;
-      ++calls;
+    for (int i = 0; i < K; ++i)
 #pragma unroll
-      for (int i = 0; i < K; ++i) C.lam[i] = i == 0 ? 1.f : 0.f;
-    } else {  // warm: the stored vertices' points for this G
-      float tot = 0.f;
+      for (int r = 0; r < 6; ++r) P[i][r] = 0.f;
 #pragma unroll
-      for (int i = 0; i < K; ++i)
-        if (i < C.n) {
-          point(G, b, C.V[i], c, P[i]);
-          C.lam[i] = fmaxf(C.lam[i], 0.f);
-          tot += C.lam[i];
-        } else {
-          C.lam[i] = 0.f;
-        }
-      const float it = tot > 0.f ? 1.f / tot : 0.f;
+    for (int i = 0; i < K - 1; ++i) {
+      D[i] = 0.f;
 #pragma unroll
-      for (int i = 0; i < K; ++i) C.lam[i] = i < C.n ? (tot > 0.f ? C.lam[i] * it : 1.f / C.n) : 0.f;
-      if (C.n > 1) minor(P, C);
+      for (int r = 0; r < 6; ++r) U[i][r] = 0.f;
     }
-    int& n = C.n;
-    bool capped = false;
-    int stall = 0;
+#pragma unroll
+    for (int i = 0; i < (K - 1) * (K - 2) / 2; ++i) R[i] = 0.f;
+    int n = n_io, cols = 0;  // points; columns of U, R, D that are valid for them
+    int calls = 0, guard = 0, stall = 0;
+    bool minor = false, warm = false, capped = false;
     float prev_xx = 3.4e38f;
     gap = 0.f;
-#pragma unroll 1
-    for (;;) {
+    if (n <= 0 || n > K) {
+      n = 0;
 #pragma unroll
-      for (int r = 0; r < 6; ++r) {
-        float s = 0.f;
+      for (int i = 0; i < K; ++i) lam[i] = 0.f;
+    } else {  // warm: the stored vertices' points for this G
+      float tot = 0.f;
+#pragma unroll 1
+      for (int k = 0; k < n; ++k) {
+        float q[6];
+        point(G, b, Vtx{__float_as_int(vs[k * stride]), vs[(K + k) * stride]}, c, edge, q);
 #pragma unroll
         for (int i = 0; i < K; ++i)
-          if (i < n) s = fmaf(C.lam[i], P[i][r], s);
-        x[r] = s;
+#pragma unroll
+          for (int r = 0; r < 6; ++r) P[i][r] = i == k ? q[r] : P[i][r];
       }
-      float q[6];
-      const Vtx vn = oracle(G, b, x, c, q);
-      ++calls;
-      float xx = 0.f, xq = 0.f;
 #pragma unroll
-      for (int r = 0; r < 6; ++r) {
-        xx = fmaf(x[r], x[r], xx);
-        xq = fmaf(x[r], q[r], xq);
+      for (int i = 0; i < K; ++i) {
+        lam[i] = i < n ? fmaxf(lam[i], 0.f) : 0.f;
+        if (i < n) tot += lam[i];
       }
-      gap = xx - xq;
-      if (gap <= fmaf(1e-5f, xx, 1e-7f) || n >= K) break;
-      // |x| falls at every major step in exact arithmetic; three steps
-      // without a relative 1e-6 decrease: float32 resolution is reached
-      stall = xx > prev_xx * (1.f - 1e-6f) ? stall + 1 : 0;
-      prev_xx = xx;
-      if (stall >= 3) break;
-      bool seen = false;  // the oracle cycles back to a vertex of the set
+      const float it = tot > 0.f ? 1.f / tot : 0.f;
 #pragma unroll
-      for (int i = 0; i < K; ++i)
-        if (i < n) seen = seen || (C.V[i].code == vn.code && C.V[i].frac == vn.frac);
-      if (seen) break;
-      if (calls >= max_calls) {
-        capped = true;
-        break;
-      }
-      // add the vertex with weight 0 (slot n), then minor cycles
-#pragma unroll
-      for (int i = 0; i < K; ++i)
-        if (i == n) {
-          C.V[i] = vn;
-#pragma unroll
-          for (int r = 0; r < 6; ++r) P[i][r] = q[r];
-          C.lam[i] = 0.f;
-        }
-      ++n;
-      if (!minor(P, C)) {  // the newcomer is dependent: the current point stands
+      for (int i = 0; i < K; ++i) lam[i] = i < n ? (tot > 0.f ? lam[i] * it : 1.f / n) : 0.f;
+      minor = warm = n > 1;
+    }
+#pragma unroll 1
+    for (;;) {
+      if (!minor) {
+        float x[6], q[6];
 #pragma unroll
         for (int r = 0; r < 6; ++r) {
           float s = 0.f;
 #pragma unroll
           for (int i = 0; i < K; ++i)
-            if (i < n) s = fmaf(C.lam[i], P[i][r], s);
-          x[r] = s;
+            if (i < n) s = fmaf(lam[i], P[i][r], s);
+          x[r] = n == 0 ? -b[r] : s;  // cold: the oracle's vertex at y = 0 (x = -b)
         }
-        break;
+        const Vtx vn = oracle(G, b, x, c, edge, q);
+        ++calls;
+        if (n > 0) {
+          float xx = 0.f, xq = 0.f;
+#pragma unroll
+          for (int r = 0; r < 6; ++r) {
+            xx = fmaf(x[r], x[r], xx);
+            xq = fmaf(x[r], q[r], xq);
+          }
+          gap = xx - xq;
+          if (gap <= fmaf(1e-5f, xx, 1e-7f) || n >= K) break;
+          // |x| falls at every major step in exact arithmetic; three steps
+          // without a relative 1e-6 decrease: float32 resolution is reached
+          stall = xx > prev_xx * (1.f - 1e-6f) ? stall + 1 : 0;
+          prev_xx = xx;
+          if (stall >= 3) break;
+          bool seen = false;  // the oracle cycles back to a vertex of the set
+#pragma unroll 1
+          for (int i = 0; i < n; ++i)
+            seen = seen || (__float_as_int(vs[i * stride]) == vn.code && vs[(K + i) * stride] == vn.frac);
+          if (seen) break;
+          if (calls >= max_calls) {
+            capped = true;
+            break;
+          }
+          minor = true;
+          guard = 0;
+        }
+        // add the vertex with weight 0 (slot n; the first one with weight 1)
+#pragma unroll
+        for (int i = 0; i < K; ++i) {
+#pragma unroll
+          for (int r = 0; r < 6; ++r) P[i][r] = i == n ? q[r] : P[i][r];
+          lam[i] = i == n ? (n == 0 ? 1.f : 0.f) : lam[i];
+        }
+        vs[n * stride] = __int_as_float(vn.code);
+        vs[(K + n) * stride] = vn.frac;
+        ++n;
+      }
+      if (minor) {
+        // the columns of D's QR factors that are not valid any more; false
+        // when the differences are (numerically) dependent
+        float sc = 1.f;
+#pragma unroll
+        for (int i = 0; i < K; ++i)
+          if (i < n)
+#pragma unroll
+            for (int r = 0; r < 6; ++r) sc = fmaxf(sc, fabsf(P[i][r]));
+        const float tiny = 1e-6f * sc;
+        bool full = true;
+#pragma unroll
+        for (int j = 0; j < K - 1; ++j)
+          if (j < cols) full = full && D[j] > tiny;  // sc may have grown since
+#pragma unroll 1
+        while (full && cols < n - 1) {
+          float u[6], rc[K - 2];
+#pragma unroll
+          for (int r = 0; r < 6; ++r) u[r] = P[1][r];
+#pragma unroll
+          for (int i = 2; i < K; ++i)
+#pragma unroll
+            for (int r = 0; r < 6; ++r) u[r] = pick(i == cols + 1, P[i][r], u[r]);
+#pragma unroll
+          for (int r = 0; r < 6; ++r) u[r] = u[r] - P[0][r];
+#pragma unroll
+          for (int i = 0; i < K - 2; ++i) rc[i] = 0.f;
+#pragma unroll
+          for (int pass = 0; pass < 2; ++pass)
+#pragma unroll
+            for (int i = 0; i < K - 2; ++i)
+              if (i < cols) {
+                float d = 0.f;
+#pragma unroll
+                for (int r = 0; r < 6; ++r) d = fmaf(U[i][r], u[r], d);
+                rc[i] += d;
+#pragma unroll
+                for (int r = 0; r < 6; ++r) u[r] = fmaf(-d, U[i][r], u[r]);
+              }
+          float nn = 0.f;
+#pragma unroll
+          for (int r = 0; r < 6; ++r) nn = fmaf(u[r], u[r], nn);
+          const float rjj = sqrtf(nn);
+          if (!(rjj > tiny)) {
+            full = false;
+            break;
+          }
+          const float inv = 1.f / rjj;
+#pragma unroll
+          for (int j = 0; j < K - 1; ++j) {
+            D[j] = j == cols ? rjj : D[j];
+#pragma unroll
+            for (int r = 0; r < 6; ++r) U[j][r] = j == cols ? u[r] * inv : U[j][r];
+#pragma unroll
+            for (int i = 0; i < j; ++i) R[ri(i, j)] = j == cols ? rc[i] : R[ri(i, j)];
+          }
+          ++cols;
+        }
+        if (!full) {  // dependent points: drop the last one, keep the current weights
+          --n;
+          cols = 0;
+          float tot = 0.f;
+#pragma unroll
+          for (int i = 0; i < K; ++i) tot += i < n ? lam[i] : 0.f;
+          const float it = tot > 0.f ? 1.f / tot : 0.f;
+#pragma unroll
+          for (int i = 0; i < K; ++i) lam[i] = i < n ? (tot > 0.f ? lam[i] * it : (i == 0 ? 1.f : 0.f)) : 0.f;
+          if (!warm) break;  // the newcomer is dependent: the current point stands
+          minor = warm = false;
+        } else {
+          // weights of the affine hull's nearest point (sum 1)
+          float al[K];
+#pragma unroll
+          for (int j = K - 2; j >= 0; --j) {
+            float s = 0.f;
+#pragma unroll
+            for (int r = 0; r < 6; ++r) s = fmaf(-U[j][r], P[0][r], s);
+#pragma unroll
+            for (int k = K - 2; k > j; --k)
+              if (k + 1 < n) s = fmaf(-R[ri(j, k)], al[k + 1], s);
+            al[j + 1] = j + 1 < n ? s / D[j] : 0.f;
+          }
+          float a0 = 1.f;
+#pragma unroll
+          for (int j = 0; j < K - 1; ++j)
+            if (j + 1 < n) a0 -= al[j + 1];
+          al[0] = a0;
+          bool inside = true;
+#pragma unroll
+          for (int i = 0; i < K; ++i)
+            if (i < n) inside = inside && al[i] > 0.f;
+          if (inside) {
+#pragma unroll
+            for (int i = 0; i < K; ++i) lam[i] = i < n ? al[i] : 0.f;
+            minor = warm = false;
+          } else {
+            float th = 1.f;
+            int drop = -1;
+#pragma unroll
+            for (int i = 0; i < K; ++i)
+              if (i < n && al[i] <= 0.f) {
+                const float den = lam[i] - al[i];
+                const float ti = den > 0.f ? lam[i] / den : 0.f;
+                if (drop < 0 || ti < th) th = ti, drop = i;
+              }
+            float tot = 0.f;
+#pragma unroll
+            for (int i = 0; i < K; ++i)
+              if (i < n) {
+                lam[i] = i == drop ? 0.f : fmaxf(fmaf(th, al[i] - lam[i], lam[i]), 0.f);
+                tot += lam[i];
+              }
+            // compact: move the last point into the dropped slot
+            const int last = n - 1;
+            if (drop >= 0 && drop != last) {
+              float pl[6], ll = 0.f;
+#pragma unroll
+              for (int r = 0; r < 6; ++r) pl[r] = 0.f;
+#pragma unroll
+              for (int i = 1; i < K; ++i) {
+                ll = i == last ? lam[i] : ll;
+#pragma unroll
+                for (int r = 0; r < 6; ++r) pl[r] = pick(i == last, P[i][r], pl[r]);
+              }
+#pragma unroll
+              for (int i = 0; i < K - 1; ++i) {
+                lam[i] = i == drop ? ll : lam[i];
+#pragma unroll
+                for (int r = 0; r < 6; ++r) P[i][r] = i == drop ? pl[r] : P[i][r];
+              }
+              vs[drop * stride] = vs[last * stride];
+              vs[(K + drop) * stride] = vs[(K + last) * stride];
+              cols = min(cols, max(drop - 1, 0));  // column j is the difference p_{j+1} - p_0
+            }
+            --n;
+            cols = min(cols, n - 1);
+            const float it = tot > 0.f ? 1.f / tot : 0.f;
+#pragma unroll
+            for (int i = 0; i < K; ++i) lam[i] = i < n ? lam[i] * it : 0.f;
+            if (n == 1) {
+              lam[0] = 1.f;
+              minor = warm = false;
+            } else if (++guard >= 2 * K) {
+              minor = warm = false;
+            }
+          }
+        }
       }
     }
 #pragma unroll
     for (int a = 0; a < NV; ++a) y[a] = 0.f;
 #pragma unroll
     for (int i = 0; i < K; ++i)
-      if (i < n) accumulate_y(C.V[i], C.lam[i], c, y);
+      if (i < n) accumulate_y(Vtx{__float_as_int(vs[i * stride]), vs[(K + i) * stride]}, lam[i], c, edge, y);
     Q = 0.f;
 #pragma unroll
     for (int r = 0; r < 6; ++r) {
-      float s = c.beta * t[r];
+      float s = __fmul_rn(c.beta, t[r]);
 #pragma unroll
       for (int a = 0; a < NV; ++a) s = fmaf(-G[r * NV + a], y[a], s);
       Q = fmaf(s, s, Q);
     }
+    n_io = n;
     return capped ? -calls : calls;
   }
 };

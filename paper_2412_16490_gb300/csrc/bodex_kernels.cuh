@@ -575,7 +575,7 @@ __global__ void __launch_bounds__(CTA_LANES, 4) qp_solve_kernel(const float* __r
 // Q - Q*), z = A y clamped to the row bounds, lam = 0 (the method gives no
 // multipliers); BODEX_ST_NOT_CONVERGED when the oracle-call cap stopped it.
 template <int M>
-__global__ void __launch_bounds__(128) qp_exact_kernel(const float* __restrict__ Gin, int B,
+__global__ void __launch_bounds__(CTA_LANES, 4) qp_exact_kernel(const float* __restrict__ Gin, int B,
                                                        const float* __restrict__ T, int S, AdmmCfg cfg, float* y_out,
                                                        float* z_out, float* l_out, float* Qout, int32_t* iters_out,
                                                        int32_t* status_out, float* res_out) {
@@ -584,18 +584,22 @@ __global__ void __launch_bounds__(128) qp_exact_kernel(const float* __restrict__
   const int GPB = blockDim.x / S;
   const size_t g0 = (size_t)blockIdx.x * GPB;
   const int ng = (int)min((size_t)GPB, (size_t)B - g0);
-  for (int e = threadIdx.x; e < ng * 6 * NV; e += blockDim.x) smem[e] = Gin[g0 * 6 * NV + e];
+  float* const edge = smem;                            // edge table, vertices [VW][threads], then G
+  float* const vs = edge + ExactQP<M>::EDGE_WORDS;
+  float* const Gs = vs + ExactQP<M>::VW * blockDim.x;
+  ExactQP<M>::fill_edges(edge);
+  for (int e = threadIdx.x; e < ng * 6 * NV; e += blockDim.x) Gs[e] = Gin[g0 * 6 * NV + e];
   __syncthreads();
   const int gl = threadIdx.x / S, j = threadIdx.x % S;
   if (gl >= ng) return;
   const size_t q = (g0 + gl) * S + j;
-  const float* G = smem + gl * 6 * NV;
+  const float* G = Gs + gl * 6 * NV;
   float t[6], y[NV], Q, gap;
 #pragma unroll
   for (int r = 0; r < 6; ++r) t[r] = T[j * 6 + r];
-  typename ExactQP<M>::Corral C;
-  C.n = 0;
-  const int ret = ExactQP<M>::solve(G, t, cfg, cfg.iters, C, y, Q, gap);
+  int n = 0;
+  float lam[ExactQP<M>::K];
+  const int ret = ExactQP<M>::solve(G, t, cfg, edge, cfg.iters, n, lam, vs + threadIdx.x, blockDim.x, y, Q, gap);
   const int calls = ret < 0 ? -ret : ret;
   bool fin = isfinite(Q);
 #pragma unroll
@@ -646,6 +650,8 @@ __global__ void __launch_bounds__(QP_FINISH_THREADS) qp_finish_kernel(const floa
   constexpr int NV = 3 * M;
   __shared__ int list[QP_FINISH_RANGE];
   __shared__ int count;
+  __shared__ float edge[ExactQP<M, false>::EDGE_WORDS], vs[ExactQP<M, false>::VW * QP_FINISH_THREADS];
+  ExactQP<M, false>::fill_edges(edge);
   const size_t n = (size_t)B * S, q0 = (size_t)blockIdx.x * QP_FINISH_RANGE;
   if (threadIdx.x == 0) count = 0;
   __syncthreads();
@@ -668,9 +674,9 @@ __global__ void __launch_bounds__(QP_FINISH_THREADS) qp_finish_kernel(const floa
     float t[6], y[NV], Q, gap;
 #pragma unroll
     for (int r = 0; r < 6; ++r) t[r] = T[j * 6 + r];
-    typename ExactQP<M>::Corral C;
-    C.n = 0;
-    if (ExactQP<M>::solve(G, t, cfg, 64, C, y, Q, gap) < 0) continue;
+    int m = 0;
+    float lam[ExactQP<M, false>::K];
+    if (ExactQP<M, false>::solve(G, t, cfg, edge, 64, m, lam, vs + threadIdx.x, QP_FINISH_THREADS, y, Q, gap) < 0) continue;
 #pragma unroll
     for (int a = 0; a < NV; ++a) y_io[q * NV + a] = y[a];
     Qout[q] = Q;
@@ -820,6 +826,9 @@ __device__ __forceinline__ void fused_cta(const FusedArgs& A, int cta, int GPB, 
   float t[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
   if (active)
     for (int r = 0; r < 6; ++r) t[r] = A.T[lane * 6 + r];
+  // the exact solver's edge table, in the first grasp's K^-1 block (no K^-1 there)
+  float* const edge = smem + L::HAND_WORDS;
+  if (CONE == CONE_EXACT) ExactQP<M>::fill_edges(edge);
   __syncthreads();
 
   const float lb1 = log2f(A.b1), lb2 = log2f(A.b2);
@@ -890,26 +899,29 @@ __device__ __forceinline__ void fused_cta(const FusedArgs& A, int cta, int GPB, 
       // the exact lower level: each lane solves its QP from the corral its
       // previous step left (cold at the first step of a run)
       if (active && !A.dfc && MODE != MODE_ADJOINT) {
-        typename ExactQP<M>::Corral C;
-        C.n = 0;
+        constexpr int K = ExactQP<M>::K;
+        int n = 0;
+        float lam[K];
+        // the vertices live in this lane's output record, written only after the solve
+        float* const vs = per + L::oRY + lane * L::RYW;
         if (A.qw) {
-          C.n = __float_as_int(A.qw[q]);
+          n = __float_as_int(A.qw[q]);
 #pragma unroll
-          for (int i = 0; i < ExactQP<M>::K; ++i) {
-            C.V[i].code = __float_as_int(A.qw[(1 + i) * NQ + q]);
-            C.V[i].frac = A.qw[(8 + i) * NQ + q];
-            C.lam[i] = A.qw[(15 + i) * NQ + q];
+          for (int i = 0; i < K; ++i) {
+            vs[i] = A.qw[(1 + i) * NQ + q];
+            vs[K + i] = A.qw[(8 + i) * NQ + q];
+            lam[i] = A.qw[(15 + i) * NQ + q];
           }
         }
         float Qx, gap;
-        const int ret = ExactQP<M>::solve(Gs, t, cfg, cfg.iters, C, y, Qx, gap);
+        const int ret = ExactQP<M>::solve(Gs, t, cfg, edge, cfg.iters, n, lam, vs, 1, y, Qx, gap);
         if (A.qw) {
-          A.qw[q] = __int_as_float(C.n);
+          A.qw[q] = __int_as_float(n);
 #pragma unroll
-          for (int i = 0; i < ExactQP<M>::K; ++i) {
-            A.qw[(1 + i) * NQ + q] = __int_as_float(C.V[i].code);
-            A.qw[(8 + i) * NQ + q] = C.V[i].frac;
-            A.qw[(15 + i) * NQ + q] = C.lam[i];
+          for (int i = 0; i < K; ++i) {
+            A.qw[(1 + i) * NQ + q] = vs[i];
+            A.qw[(8 + i) * NQ + q] = vs[K + i];
+            A.qw[(15 + i) * NQ + q] = lam[i];
           }
         }
         if (step == A.n_steps - 1) atomicMax(reinterpret_cast<int*>(sc + 2), __float_as_int(fmaxf(gap, 0.f)));
@@ -1161,7 +1173,7 @@ __device__ __forceinline__ void fused_cta(const FusedArgs& A, int cta, int GPB, 
 }
 
 template <int M, int MODE, int CONE, bool ADAPT>
-__global__ void __launch_bounds__(CTA_LANES, CONE == CONE_EXACT ? 2 : 4) fused_kernel(FusedArgs A) {
+__global__ void __launch_bounds__(CTA_LANES, 4) fused_kernel(FusedArgs A) {
   extern __shared__ __align__(16) float smem[];
   fused_cta<M, MODE, CONE, ADAPT>(A, blockIdx.x, A.gpb, smem);
 }
@@ -1212,7 +1224,7 @@ __device__ __forceinline__ void multi_item(const MultiArgs& A, int w, float* sme
 }
 
 template <bool ADAPT, bool EXACT = false, bool PULL = false>
-__global__ void __launch_bounds__(CTA_LANES, EXACT ? 2 : 4) multi_kernel(const __grid_constant__ MultiArgs A) {
+__global__ void __launch_bounds__(CTA_LANES, 4) multi_kernel(const __grid_constant__ MultiArgs A) {
   extern __shared__ __align__(16) float smem[];
   if constexpr (!PULL) {
     multi_item<ADAPT, EXACT>(A, (int)blockIdx.x, smem);  // one item per CTA, no loop
@@ -1324,8 +1336,8 @@ inline int run_qp(const float* G, int B, const float* T, int s, const AdmmCfg& c
            float* lam, float* Q, int32_t* iters, int32_t* status, float* res, cudaStream_t st) {
   if (B == 0) return BODEX_OK;
   if (cfg.solver == BODEX_QP_EXACT) {
-    const int gpb = std::max(1, 128 / s);
-    const size_t bytes = 4u * (size_t)gpb * 6 * 3 * M;
+    const int gpb = std::max(1, CTA_LANES / s);
+    const size_t bytes = 4u * (size_t)(ExactQP<M>::EDGE_WORDS + gpb * (s * ExactQP<M>::VW + 6 * 3 * M));
     qp_exact_kernel<M><<<(B + gpb - 1) / gpb, gpb * s, bytes, st>>>(G, B, T, s, cfg, y, z, lam, Q, iters, status,
                                                                     res);
     return launch_err("qp_exact_kernel launch");
