@@ -86,33 +86,50 @@ struct bodex_state_s {
 };
 
 // ============================================================================ kernel: FK + contacts + G
+// One thread per contact, FkTile<M>::GPB grasps a block: poses come in and
+// the grasp matrices (18 floats a contact, spread over six rows) go out
+// through shared memory, so that both are coalesced.  With one thread per
+// grasp, walking its contacts in turn and storing 90 floats at a stride of
+// 360 bytes, a batch of 16,384 five-finger poses was 512 warps of mostly
+// waiting threads: 28 us.
 template <int M>
-__global__ void __launch_bounds__(128) fk_contacts_kernel(const HandDev* __restrict__ hand, ObjDev obj,
+struct FkTile {
+  static constexpr int THREADS = 128, GPB = THREADS / M;
+};
+
+template <int M>
+__global__ void __launch_bounds__(FkTile<M>::THREADS) fk_contacts_kernel(const HandDev* __restrict__ hand, ObjDev obj,
                                                           const float* __restrict__ x, int B, float* c_w,
                                                           float* p_out, float* n_out, float* phi_out, float* G_out,
                                                           int32_t* cell_out, int32_t* status_out) {
+  constexpr int NV = 3 * M, GPB = FkTile<M>::GPB;
   __shared__ __align__(16) float hs[Lay<M>::HAND_WORDS];
+  __shared__ float xs[GPB * MAXD];
+  __shared__ float Gs[GPB * 6 * NV];
+  __shared__ int stat[GPB];
   copy_hand_to_smem(hand, hs);
-  __syncthreads();
   const HandDev& H = *reinterpret_cast<const HandDev*>(hs);
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= B) return;
-  constexpr int NV = 3 * M;
-  const int D = H.D;
-  float xl[MAXD];
-  int st = 0;
-  for (int k = 0; k < D; ++k) {
-    xl[k] = x[(size_t)b * D + k];
-    if (!isfinite(xl[k])) st |= BODEX_ST_NONFINITE;
+  const int D = __ldg(&hand->D);
+  const int b0 = blockIdx.x * GPB, ng = min(GPB, B - b0);
+  if ((int)threadIdx.x < GPB) stat[threadIdx.x] = 0;
+  __syncthreads();
+  for (int e = threadIdx.x; e < ng * D; e += blockDim.x) {
+    const float v = x[(size_t)b0 * D + e];
+    xs[e] = v;
+    if (!isfinite(v)) atomicOr(stat + e / D, BODEX_ST_NONFINITE);
   }
-  float Gl[6 * NV];
-  for (int i = 0; i < M; ++i) {
+  __syncthreads();
+  const int gl = threadIdx.x / M, i = threadIdx.x % M;
+  if (gl < ng) {
+    const int b = b0 + gl;
     float c[3];
-    fk_contact(H, i, xl, c, nullptr);
+    fk_contact(H, i, xs + gl * D, c, nullptr);
     const ContactGeo k = contact_geometry(obj, c);
+    int st = 0;
     if (k.degenerate) st |= BODEX_ST_DEGENERATE_NORMAL;
     if (!finite3(k.p) || !finite3(k.n) || !isfinite(k.phi)) st |= BODEX_ST_NONFINITE;
-    write_G_block(k, i, NV, Gl);
+    if (st) atomicOr(stat + gl, st);
+    write_G_block(k, i, NV, Gs + gl * 6 * NV);
     const size_t o = ((size_t)b * M + i) * 3;
     const float gc[3] = {obj.gcx, obj.gcy, obj.gcz};
     for (int a = 0; a < 3; ++a) {
@@ -123,9 +140,10 @@ __global__ void __launch_bounds__(128) fk_contacts_kernel(const HandDev* __restr
     }
     if (phi_out) phi_out[(size_t)b * M + i] = k.phi;
   }
+  __syncthreads();
   if (G_out)
-    for (int e = 0; e < 6 * NV; ++e) G_out[(size_t)b * 6 * NV + e] = Gl[e];
-  if (status_out) status_out[b] = st;
+    for (int e = threadIdx.x; e < ng * 6 * NV; e += blockDim.x) G_out[(size_t)b0 * 6 * NV + e] = Gs[e];
+  if (status_out && (int)threadIdx.x < ng) status_out[b0 + threadIdx.x] = stat[threadIdx.x];
 }
 
 // ============================================================================ kernel: refinement epilogue
@@ -136,8 +154,13 @@ __global__ void __launch_bounds__(128) fk_contacts_kernel(const HandDev* __restr
 //   E = w_d sum |c^{f'} - (p^f + delta n_out)|^2 + w_qp sum |c^{f'} - p^c|^2
 // with p^f, n_out and the coarse-stage points p^c treated as constants.
 // delta is the pre-grasp margin (Sec. IV-D): 1 cm in the fine stage, 0 in
-// the final one.  One CTA holds RF_GPB grasps x 8 lanes; lanes 0..m-1 own a
-// contact, all lanes share the gradient assembly and Adam.
+// the final one.  One warp per grasp and RF_GPB warps a block, with no block
+// barrier between steps: lanes 0..m-1 own a contact's kinematics and adjoint,
+// all 32 lanes share each fingertip's samples (the queries are most of the
+// work: 160 a grasp and step), the gradient assembly and Adam.  With eight
+// lanes a grasp and each contact's samples walked by one of them, a step of
+// 4096 grasps was bound by the latency of 32 queries in a row on 6.7 warps an
+// SM.
 struct RefineArgs {
   const HandDev* hand;
   const float* tips;
@@ -155,18 +178,57 @@ struct RefineArgs {
   int32_t* status;
 };
 
-constexpr int RF_LANES = 8, RF_GPB = 16;
+constexpr int RF_GPB = 4;  // grasps (warps) per block of the refinement and metrics kernels
+
+// The fingertip sample with the smallest phi over the warp, lowest index on
+// ties (0 if none compares below infinity): T is the contact's link frame.
+// phi receives the smallest value (infinity if none).
+__device__ __forceinline__ int lowest_sample(const Tf& T, const float* __restrict__ tip, int S, const ObjDev& obj,
+                                             float& phi) {
+  const int lane = threadIdx.x % 32;
+  float best = INFINITY;
+  int kbest = 0;
+  for (int k = lane; k < S; k += 32) {
+    const float sk[3] = {__ldg(tip + 3 * k), __ldg(tip + 3 * k + 1), __ldg(tip + 3 * k + 2)};
+    float ck[3];
+    tf_point(T, sk, ck);
+    const float ph = sdf_query(obj, ck).phi;
+    if (ph < best) {
+      best = ph;
+      kbest = k;
+    }
+  }
+#pragma unroll
+  for (int off = 16; off >= 1; off >>= 1) {
+    const float b2 = __shfl_xor_sync(0xffffffffu, best, off);
+    const int k2 = __shfl_xor_sync(0xffffffffu, kbest, off);
+    if (b2 < best || (b2 == best && k2 < kbest)) {
+      best = b2;
+      kbest = k2;
+    }
+  }
+  phi = best;
+  return best < INFINITY ? kbest : 0;
+}
+
+// A link frame in shared memory, 12 words.
+__device__ __forceinline__ void load_frame(const float* f, Tf& T) {
+#pragma unroll
+  for (int e = 0; e < 9; ++e) T.R[e] = f[e];
+  T.t[0] = f[9];
+  T.t[1] = f[10];
+  T.t[2] = f[11];
+}
 
 template <int M>
-__global__ void __launch_bounds__(RF_LANES * RF_GPB) refine_kernel(RefineArgs A) {
+__global__ void __launch_bounds__(32 * RF_GPB) refine_kernel(RefineArgs A) {
   constexpr int HW = Lay<M>::HAND_WORDS;
   constexpr int CBW = 6 + MAXCHAIN;
-  constexpr int PER = align4(3 * MAXD + M * CBW + M * MAXCHAIN * 6 + M + 4);
+  constexpr int PER = align4(3 * MAXD + M * CBW + M * MAXCHAIN * 6 + M * 12 + M + 4);
   __shared__ __align__(16) float smem[HW + RF_GPB * PER];
   copy_hand_to_smem(A.hand, smem);
-  const int gl = threadIdx.x / RF_LANES, lane = threadIdx.x % RF_LANES;
+  const int gl = threadIdx.x / 32, lane = threadIdx.x % 32;
   const int b = blockIdx.x * RF_GPB + gl;
-  const bool active = b < A.B;
   const HandDev& H = *reinterpret_cast<const HandDev*>(smem);
   float* per = smem + HW + gl * PER;
   float* xs = per;
@@ -174,38 +236,40 @@ __global__ void __launch_bounds__(RF_LANES * RF_GPB) refine_kernel(RefineArgs A)
   float* avs = per + 2 * MAXD;
   float* cb = per + 3 * MAXD;
   float* jwall = cb + M * CBW;
-  float* Ei = jwall + M * MAXCHAIN * 6;
+  float* frames = jwall + M * MAXCHAIN * 6;
+  float* Ei = frames + M * 12;
   int* stat = reinterpret_cast<int*>(Ei + M);
   __syncthreads();
+  if (b >= A.B) return;  // whole warps; no block barrier below
   const int D = H.D, S = H.S;
-  if (active) {
-    for (int k = lane; k < D; k += RF_LANES) {
-      xs[k] = A.x[(size_t)b * D + k];
-      ams[k] = A.am[(size_t)b * D + k];
-      avs[k] = A.av[(size_t)b * D + k];
-    }
-    if (lane == 0) *stat = 0;
+  for (int k = lane; k < D; k += 32) {
+    xs[k] = A.x[(size_t)b * D + k];
+    ams[k] = A.am[(size_t)b * D + k];
+    avs[k] = A.av[(size_t)b * D + k];
   }
-  __syncthreads();
+  if (lane == 0) *stat = 0;
+  __syncwarp();
   int kbest = 0;
   for (int step = 0; step < A.n_steps; ++step) {
-    if (active && lane < M) {
+    const float* jw = jwall + (lane < M ? lane : 0) * MAXCHAIN * 6;
+    if (lane < M) {
       Tf T;
-      float* jw = jwall + lane * MAXCHAIN * 6;
-      fk_link(H, lane, xs, T, jw);
+      fk_link(H, lane, xs, T, jwall + lane * MAXCHAIN * 6);
+      store_frame(T, frames + 12 * lane);
+    }
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < M; ++i) {
+      Tf T;
+      load_frame(frames + 12 * i, T);
+      float phi;
+      const int k = lowest_sample(T, A.tips + (size_t)i * S * 3, S, A.obj, phi);
+      if (lane == i) kbest = k;
+    }
+    if (lane < M) {
+      Tf T;
+      load_frame(frames + 12 * lane, T);
       const float* tip = A.tips + (size_t)lane * S * 3;
-      float best = INFINITY;
-      kbest = 0;
-      for (int k = 0; k < S; ++k) {
-        const float sk[3] = {__ldg(tip + 3 * k), __ldg(tip + 3 * k + 1), __ldg(tip + 3 * k + 2)};
-        float ck[3];
-        tf_point(T, sk, ck);
-        const float ph = sdf_query(A.obj, ck).phi;
-        if (ph < best) {
-          best = ph;
-          kbest = k;
-        }
-      }
       const float sk[3] = {__ldg(tip + 3 * kbest), __ldg(tip + 3 * kbest + 1), __ldg(tip + 3 * kbest + 2)};
       float cf[3];
       tf_point(T, sk, cf);
@@ -244,8 +308,8 @@ __global__ void __launch_bounds__(RF_LANES * RF_GPB) refine_kernel(RefineArgs A)
         c[6 + kk] = dEdc[0] * v[0] + dEdc[1] * v[1] + dEdc[2] * v[2];
       }
     }
-    __syncthreads();
-    if (active) {
+    __syncwarp();
+    {
       const int tstep = A.t0 + step + 1;
       const float c1 = 1.f - exp2f((float)tstep * log2f(A.b1)), c2 = 1.f - exp2f((float)tstep * log2f(A.b2));
       if (lane == 0 && A.E) {
@@ -253,7 +317,7 @@ __global__ void __launch_bounds__(RF_LANES * RF_GPB) refine_kernel(RefineArgs A)
         for (int i = 0; i < M; ++i) e += Ei[i];
         per[PER - 1] = e;
       }
-      for (int k = lane; k < D; k += RF_LANES) {
+      for (int k = lane; k < D; k += 32) {
         float g = 0.f;
         if (k < 6) {
           for (int i = 0; i < M; ++i) g += cb[i * CBW + k];
@@ -272,10 +336,9 @@ __global__ void __launch_bounds__(RF_LANES * RF_GPB) refine_kernel(RefineArgs A)
         xs[k] = fminf(fmaxf(xn, H.qmin[k]), H.qmax[k]);
       }
     }
-    __syncthreads();
+    __syncwarp();
   }
-  if (!active) return;
-  for (int k = lane; k < D; k += RF_LANES) {
+  for (int k = lane; k < D; k += 32) {
     A.x[(size_t)b * D + k] = xs[k];
     A.am[(size_t)b * D + k] = ams[k];
     A.av[(size_t)b * D + k] = avs[k];
@@ -290,8 +353,10 @@ __global__ void __launch_bounds__(RF_LANES * RF_GPB) refine_kernel(RefineArgs A)
 // ============================================================================ kernel: contact metrics
 // Contact Distance Consistency (Sec. V-B): d_i = the signed distance of
 // fingertip i, the smallest phi over its surface samples (phi(c_i) - alpha
-// for a hand without samples); cdc = max_i d_i - min_i d_i.  Eight lanes per
-// grasp, lane i < m owns finger i; the spread is reduced across the lanes.
+// for a hand without samples); cdc = max_i d_i - min_i d_i.  One warp per
+// grasp: lanes 0..m-1 place their links, then the warp shares each finger's
+// samples (with one lane a finger, walking its 32 samples: 59 us for 16,384
+// five-finger poses).
 struct MetricsArgs {
   const HandDev* hand;
   const float* tips;  // [m, S, 3] or null
@@ -303,50 +368,53 @@ struct MetricsArgs {
 };
 
 template <int M>
-__global__ void __launch_bounds__(RF_LANES * RF_GPB) metrics_kernel(MetricsArgs A) {
+__global__ void __launch_bounds__(32 * RF_GPB) metrics_kernel(MetricsArgs A) {
   constexpr int HW = Lay<M>::HAND_WORDS;
-  constexpr int XW = align4(MAXD);
-  __shared__ __align__(16) float smem[HW + RF_GPB * XW];
+  constexpr int PER = align4(MAXD) + 12 * M;
+  __shared__ __align__(16) float smem[HW + RF_GPB * PER];
   copy_hand_to_smem(A.hand, smem);
-  const int gl = threadIdx.x / RF_LANES, lane = threadIdx.x % RF_LANES;
+  const int gl = threadIdx.x / 32, lane = threadIdx.x % 32;
   const int b = blockIdx.x * RF_GPB + gl;
-  const bool active = b < A.B;
   const HandDev& H = *reinterpret_cast<const HandDev*>(smem);
-  float* xs = smem + HW + gl * XW;
+  float* xs = smem + HW + gl * PER;
+  float* frames = xs + align4(MAXD);
   __syncthreads();
+  if (b >= A.B) return;  // whole warps; no block barrier below
   const int D = H.D, S = A.tips ? H.S : 0;
-  if (active)
-    for (int k = lane; k < D; k += RF_LANES) xs[k] = A.x[(size_t)b * D + k];
-  __syncthreads();
-  const bool mine = active && lane < M;
-  float d = 0.f;
-  if (mine) {
+  for (int k = lane; k < D; k += 32) xs[k] = A.x[(size_t)b * D + k];
+  __syncwarp();
+  if (lane < M) {
     Tf T;
     fk_link(H, lane, xs, T, nullptr);
-    if (S > 0) {
-      const float* tip = A.tips + (size_t)lane * S * 3;
-      d = INFINITY;
-      for (int k = 0; k < S; ++k) {
-        const float sk[3] = {__ldg(tip + 3 * k), __ldg(tip + 3 * k + 1), __ldg(tip + 3 * k + 2)};
-        float ck[3];
-        tf_point(T, sk, ck);
-        d = fminf(d, sdf_query(A.obj, ck).phi);
-      }
-    } else {
-      float c[3];
-      tf_point(T, H.clocal[lane], c);
-      d = sdf_query(A.obj, c).phi - H.alpha;
-    }
-    A.d[(size_t)b * M + lane] = d;
+    store_frame(T, frames + 12 * lane);
   }
-  // spread over the grasp's fingers (all lanes of the 8-lane group take part)
-  float lo = mine ? d : INFINITY, hi = mine ? d : -INFINITY;
+  __syncwarp();
+  float d = 0.f;
+  if (S > 0) {
 #pragma unroll
-  for (int off = RF_LANES / 2; off >= 1; off >>= 1) {
-    lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, off, RF_LANES));
-    hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, off, RF_LANES));
+    for (int i = 0; i < M; ++i) {
+      Tf T;
+      load_frame(frames + 12 * i, T);
+      float phi;
+      (void)lowest_sample(T, A.tips + (size_t)i * S * 3, S, A.obj, phi);
+      if (lane == i) d = phi;
+    }
+  } else if (lane < M) {
+    Tf T;
+    load_frame(frames + 12 * lane, T);
+    float c[3];
+    tf_point(T, H.clocal[lane], c);
+    d = sdf_query(A.obj, c).phi - H.alpha;
   }
-  if (active && lane == 0 && A.cdc) A.cdc[b] = hi - lo;
+  if (lane < M) A.d[(size_t)b * M + lane] = d;
+  // spread over the grasp's fingers (in the lowest eight lanes)
+  float lo = lane < M ? d : INFINITY, hi = lane < M ? d : -INFINITY;
+#pragma unroll
+  for (int off = 4; off >= 1; off >>= 1) {
+    lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, off));
+    hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, off));
+  }
+  if (lane == 0 && A.cdc) A.cdc[b] = hi - lo;
 }
 
 // ============================================================================ host helpers
@@ -383,7 +451,7 @@ int run_fk(const bodex_hand_s* h, const bodex_object_s* o, const float* x, int B
            float* phi, float* G, int32_t* cell, int32_t* status, cudaStream_t st) {
   if (B == 0) return BODEX_OK;
   (void)cudaGetLastError();
-  fk_contacts_kernel<M><<<(B + 127) / 128, 128, 0, st>>>(h->dev, o->dev, x, B, c_w, p, n, phi, G, cell, status);
+  fk_contacts_kernel<M><<<(B + FkTile<M>::GPB - 1) / FkTile<M>::GPB, FkTile<M>::THREADS, 0, st>>>(h->dev, o->dev, x, B, c_w, p, n, phi, G, cell, status);
   return launch_err("fk_contacts_kernel launch");
 }
 
@@ -393,14 +461,14 @@ namespace {
 template <int M>
 int run_refine(const RefineArgs& A, cudaStream_t st) {
   (void)cudaGetLastError();
-  refine_kernel<M><<<(A.B + RF_GPB - 1) / RF_GPB, RF_LANES * RF_GPB, 0, st>>>(A);
+  refine_kernel<M><<<(A.B + RF_GPB - 1) / RF_GPB, 32 * RF_GPB, 0, st>>>(A);
   return launch_err("refine_kernel launch");
 }
 
 template <int M>
 int run_metrics(const MetricsArgs& A, cudaStream_t st) {
   (void)cudaGetLastError();
-  metrics_kernel<M><<<(A.B + RF_GPB - 1) / RF_GPB, RF_LANES * RF_GPB, 0, st>>>(A);
+  metrics_kernel<M><<<(A.B + RF_GPB - 1) / RF_GPB, 32 * RF_GPB, 0, st>>>(A);
   return launch_err("metrics_kernel launch");
 }
 }  // namespace
