@@ -1756,6 +1756,123 @@ __device__ inline int admm_solve(float* y, float* w, const float* mq, const floa
   return it;
 }
 
+// ------------------------------------------------------------------ wide form
+// The same iteration with m lanes per QP: lane ci of the group (lanes gb ..
+// gb + m - 1 of the warp) holds contact ci's rows of w, its three components
+// of y and -q, three dense rows of alpha K^-1 in registers, and a copy of
+// the sum row.  Per iteration the group exchanges the 3m right-hand-side
+// values and the m normal components by shuffles and reads no memory.  Every
+// multiply-add is the one-lane form's, in the same order (row r of the
+// product sums j = 0 .. nv-1 in both), so the iterates agree bitwise.  One
+// QP per lane is bound by the register ports at three or more warps a
+// scheduler (1.08 us an iteration for 49,152 five-contact QPs, the wide form
+// 1.24), but with one warp a scheduler its chain of some 700 instructions is
+// all latency: 0.38 us, the wide form 0.12 (four contacts 0.29 and 0.11, the
+// elliptic cone 0.89 and 0.23).
+template <int M, int CONE>
+struct Wide {
+  static constexpr int NV = 3 * M, QPW = 32 / M, WPC = CONE == CONE_SOC ? 4 : 9;
+  float K[3][NV], y[3], mq[3], w[WPC], wsum;
+
+  __device__ __forceinline__ void clear() {
+    wsum = 0.f;
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+      y[r] = mq[r] = 0.f;
+#pragma unroll
+      for (int j = 0; j < NV; ++j) K[r][j] = 0.f;
+    }
+#pragma unroll
+    for (int k = 0; k < WPC; ++k) w[k] = 0.f;
+  }
+  // rows 3ci .. 3ci+2 of the grasp's alpha K^-1 (kin: its packed triangle)
+  __device__ __forceinline__ void load_rows(const float* kin, int ci) {
+#pragma unroll
+    for (int r = 0; r < 3; ++r)
+#pragma unroll
+      for (int j = 0; j < NV; ++j) K[r][j] = kin[Admm<M>::tri(min(3 * ci + r, j), max(3 * ci + r, j))];
+  }
+  __device__ __forceinline__ void iterate(const AdmmCfg& c, float rho, int gb) {
+    const float vsum = fmaf(2.f, fmaxf(wsum, c.gamma), -wsum);
+    float rhs[3], pc[3];
+    if (CONE == CONE_SOC) soc_contact_rhs(w, vsum, y, mq, c, rho, rhs, pc);
+    else pyr_contact_rhs(w, vsum, y, mq, c, rho, rhs);
+    float yt[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+    for (int j = 0; j < NV; ++j) {
+      const float ra = __shfl_sync(0xffffffffu, rhs[j % 3], gb + j / 3);
+#pragma unroll
+      for (int r = 0; r < 3; ++r) yt[r] = fmaf(K[r][j], ra, yt[r]);
+    }
+    float sumn = 0.f;
+#pragma unroll
+    for (int i = 0; i < M; ++i) sumn += __shfl_sync(0xffffffffu, yt[0], gb + i);
+    const float al = c.alpha, bl = 1.0f - c.alpha;
+    if (CONE == CONE_SOC) soc_contact_update(w, pc, yt[0], yt[1], yt[2], c);
+    else pyr_contact_update(w, yt[0], yt[1], yt[2], c);
+    wsum = fmaf(-al, fmaxf(wsum, c.gamma), wsum + sumn);
+#pragma unroll
+    for (int r = 0; r < 3; ++r) y[r] = fmaf(bl, y[r], yt[r]);
+  }
+  // G y of the group's QP in every lane: lane ci forms row ci and the last
+  // rows go to the first lanes, each summed in column order as in g_times
+  __device__ __forceinline__ void g_times_group(const float* G, int ci, int gb, float (&gy)[6]) const {
+    constexpr int RPL = (6 + M - 1) / M;
+    float s[RPL];
+#pragma unroll
+    for (int k = 0; k < RPL; ++k) s[k] = 0.f;
+#pragma unroll
+    for (int j = 0; j < NV; ++j) {
+      const float ya = __shfl_sync(0xffffffffu, y[j % 3], gb + j / 3);
+#pragma unroll
+      for (int k = 0; k < RPL; ++k) s[k] = fmaf(G[min(ci + k * M, 5) * NV + j], ya, s[k]);
+    }
+#pragma unroll
+    for (int r = 0; r < 6; ++r) gy[r] = __shfl_sync(0xffffffffu, s[r / M], gb + r % M);
+  }
+  // The residuals of the group's QP, as admm_residuals forms them (the
+  // maxima do not depend on the order in which rows are visited).
+  template <bool SCALES>
+  __device__ __forceinline__ void residuals(const float* G, const AdmmCfg& c, float rho, int ci, int gb, float& rp,
+                                            float& rd, float* scale) const {
+    float gy[6];
+    g_times_group(G, ci, gb, gy);
+    float sumn = 0.f, np = 0.f, nd = 0.f, at[3];
+#pragma unroll
+    for (int i = 0; i < M; ++i) sumn += __shfl_sync(0xffffffffu, y[0], gb + i);
+    const float psum = fmaxf(wsum, c.gamma), dsum = wsum - psum;
+    float p = 0.f, d = 0.f;
+    if (CONE == CONE_SOC) {
+      float dl[4];
+      soc_contact_primal<SCALES>(w, y[0], y[1], y[2], c, p, np, dl);
+      at[0] = fmaf(c.mu, dl[1], dl[0]) + dsum;
+      at[1] = dl[2];
+      at[2] = dl[3];
+    } else {
+      pyr_contact_primal<SCALES>(w, y[0], y[1], y[2], c, p, np);
+      pyr_contact_atd(w, dsum, c, at);
+    }
+    p = fmaxf(p, fabsf(sumn - psum));
+#pragma unroll
+    for (int q = 0; q < 3; ++q) dual_component<NV, SCALES>(G, 3 * ci + q, gy, y[q], mq[q], at[q], c, rho, d, nd);
+    rp = rd = 0.f;
+#pragma unroll
+    for (int i = 0; i < M; ++i) {
+      rp = fmaxf(rp, __shfl_sync(0xffffffffu, p, gb + i));
+      rd = fmaxf(rd, __shfl_sync(0xffffffffu, d, gb + i));
+    }
+    if constexpr (SCALES) {
+      np = fmaxf(np, fmaxf(fabsf(sumn), fabsf(psum)));
+      scale[0] = scale[1] = 0.f;
+#pragma unroll
+      for (int i = 0; i < M; ++i) {
+        scale[0] = fmaxf(scale[0], __shfl_sync(0xffffffffu, np, gb + i));
+        scale[1] = fmaxf(scale[1], __shfl_sync(0xffffffffu, nd, gb + i));
+      }
+    }
+  }
+};
+
 // Re-expresses the iterate for a new penalty rho' (ratio = rho / rho'),
 // keeping z = Pi(w) and lam = rho (w - Pi(w)): w <- Pi(w) + ratio (w - Pi(w)).
 // Per contact (its rows: f_n and the facets, or f_n and the cone triple) and

@@ -129,15 +129,15 @@ __device__ inline void setup_kinv(bool active, int lane, int S, const float* Gs,
 // warp whose QPs all stopped waits at the barrier and issues nothing while
 // the others iterate.  A QP carries its iterate, -q, its iteration count and
 // its slot (grasp, wrench); K^-1, G and rho stay with the grasp.
-// The last QPs of a CTA (at most 32 / m) run in a wide form on warp 0: one
-// QP per m lanes, lane i holding contact i's rows, the rhs exchanged by warp
-// shuffles and each lane forming three rows of alpha K^-1 rhs from a dense
-// copy of the grasp's K^-1; the residual check is spread over the lanes
-// too.  Alone on its SM, a QP's iteration is bound by its chain of dependent
-// instructions, which the wide form shortens: the slowest QPs of a batch
-// finish sooner (the paper batch: 2.64 ms instead of 3.26 ms).  Every
-// multiply-add is the one-lane form's, in the same order (row r of the
-// product sums j = 0 .. nv-1 in both), so the iterates agree bitwise.
+// The last QPs of a CTA (at most 32 / m a warp: 18 of 96 for m = 5) run in
+// the wide form (Wide, bodex_device.cuh), m lanes each, over as few warps as
+// hold them, repacked as they finish: alone on its scheduler a QP's iteration
+// is bound by its chain of dependent instructions, and the slowest QPs run
+// thousands.  With the rows of K^-1 in registers and every warp taking
+// groups the 49,152 five-contact QPs take 1.85 ms (2.45 with the rows in
+// shared memory and the last six QPs on warp 0).  A batch small enough runs
+// in the wide form from the start (run_qp): 67 grasps of four contacts with
+// the elliptic cone 2.31 -> 1.67 ms.
 //
 // Shared memory: alpha K^-1 per grasp (stride as in the fused kernel), the
 // per-grasp block (G, Woodbury scratch, votes, rho), the parking area (one
@@ -157,25 +157,19 @@ struct LayQP {
   static constexpr int pW = align4(NV), pM = pW + align4(NC), pI = pM + align4(NV);
   static constexpr int PW0 = pI + 4;
   static constexpr int PW = (PW0 / 4) % 2 ? PW0 : PW0 + 4;
-  // wide form: QPs per warp, w rows per contact, dense K^-1 row stride
-  // (the dense row stride is an odd number of float4s, so that the lanes of
-  // a quarter-warp, which read different rows, hit distinct bank groups)
-  static constexpr int QPW = 32 / M, WPC = CONE == CONE_SOC ? 4 : 9;
-  static constexpr int NVP = (align4(NV) / 4) % 2 ? align4(NV) : align4(NV) + 4;
-  static constexpr int WIDE_PER_QP = PW + NV * NVP;  // a record and a dense K^-1 per wide QP
+  static constexpr int QPW = Wide<M, CONE>::QPW, WPC = Wide<M, CONE>::WPC;  // wide form: QPs per warp, w rows per contact
   static size_t bytes(int gpb, int s) { return 4u * ((size_t)gpb * (KS + PER) + (size_t)gpb * s * PW + 32); }
 };
 
-template <int M, int CONE>
+template <int M, int CONE, bool ADAPT>
 __global__ void __launch_bounds__(CTA_LANES, 4) qp_solve_kernel(const float* __restrict__ Gin, int B,
-                                                                const float* __restrict__ T, int S, AdmmCfg cfg,
-                                                                int warm, float* yio, float* zio, float* lio,
+                                                                const float* __restrict__ T, int S, int GPB,
+                                                                AdmmCfg cfg, int warm, float* yio, float* zio, float* lio,
                                                                 float* Qout, int32_t* iters_out, int32_t* status_out,
                                                                 float* res_out) {
   using L = LayQP<M, CONE>;
   constexpr int NV = L::NV, NC = L::NC;
   extern __shared__ __align__(16) float smem[];
-  const int GPB = blockDim.x / S;
   // setup role of this thread: lane `lane` of grasp gl of the CTA
   const int gl = threadIdx.x / S, lane = threadIdx.x % S;
   const bool role = (gl < GPB) && (blockIdx.x * GPB + gl < B);
@@ -190,7 +184,7 @@ __global__ void __launch_bounds__(CTA_LANES, 4) qp_solve_kernel(const float* __r
   }
   __syncthreads();
   setup_kinv<M>(role, lane, S, per(gl) + L::oG, per(gl) + L::oK, kin(gl), cfg);
-  const bool adaptive = cfg.eps > 0.f && cfg.adapt;  // uniform
+  constexpr bool adaptive = ADAPT;  // cfg.eps > 0 and cfg.adapt
   const int check = cfg.eps > 0.f ? cfg.check : cfg.iters;  // without a target: residuals once, at the end
   const size_t q0 = (size_t)blockIdx.x * GPB * S;         // first QP of the CTA
   // the QP this thread runs: slot p = g * S + j of the CTA (at first its own), -1 for none
@@ -215,32 +209,24 @@ __global__ void __launch_bounds__(CTA_LANES, 4) qp_solve_kernel(const float* __r
       for (int r = 0; r < NC; ++r) w[r] = 0.f;
     }
   }
-  // y, z = Pi(w), lam = rho (w - Pi(w)), Q, iterations, residuals and status of slot pp
-  auto finish = [&](int pp, float rp, float rd, bool conv) {
+  // Q, iterations, residuals and status of slot pp at the point yy
+  auto finish = [&](int pp, const float (&yy)[NV], float rp, float rd, bool conv) {
     const int g = pp / S, j = pp % S;
     const size_t q = q0 + pp;
     const float* Gg = per(g) + L::oG;
-    const float rho = per(g)[L::oRho];
     float Q = 0.f;
     bool fin = true;
 #pragma unroll
     for (int r = 0; r < 6; ++r) {
       float s = cfg.beta * T[j * 6 + r];
 #pragma unroll
-      for (int a = 0; a < NV; ++a) s = fmaf(-Gg[r * NV + a], y[a], s);
+      for (int a = 0; a < NV; ++a) s = fmaf(-Gg[r * NV + a], yy[a], s);
       Q = fmaf(s, s, Q);
     }
 #pragma unroll
     for (int a = 0; a < NV; ++a) {
-      yio[q * NV + a] = y[a];
-      fin = fin && isfinite(y[a]);
-      Q = fmaf(cfg.eps_reg * y[a], y[a], Q);  // regularised value when eps_reg > 0
-    }
-#pragma unroll
-    for (int r = 0; r < NC; ++r) {
-      const float pr = CONE == CONE_SOC ? proj_row_soc<M>(w, r, cfg.gamma) : proj_row<M>(w[r], r, cfg.gamma);
-      zio[q * NC + r] = pr;
-      lio[q * NC + r] = rho * (w[r] - pr);
+      fin = fin && isfinite(yy[a]);
+      Q = fmaf(cfg.eps_reg * yy[a], yy[a], Q);  // regularised value when eps_reg > 0
     }
     Qout[q] = Q;
     if (iters_out) iters_out[q] = it;
@@ -252,6 +238,20 @@ __global__ void __launch_bounds__(CTA_LANES, 4) qp_solve_kernel(const float* __r
     if (!fin || !isfinite(Q)) st |= BODEX_ST_NONFINITE;
     if (cfg.eps > 0.f && !conv) st |= BODEX_ST_NOT_CONVERGED;
     if (status_out) status_out[q] = st;
+  };
+  // y, z = Pi(w) and lam = rho (w - Pi(w)) of the one-lane form, then the rest
+  auto finish_lane = [&](int pp, float rp, float rd, bool conv) {
+    const size_t q = q0 + pp;
+    const float rho = per(pp / S)[L::oRho];
+#pragma unroll
+    for (int a = 0; a < NV; ++a) yio[q * NV + a] = y[a];
+#pragma unroll
+    for (int r = 0; r < NC; ++r) {
+      const float pr = CONE == CONE_SOC ? proj_row_soc<M>(w, r, cfg.gamma) : proj_row<M>(w[r], r, cfg.gamma);
+      zio[q * NC + r] = pr;
+      lio[q * NC + r] = rho * (w[r] - pr);
+    }
+    finish(pp, y, rp, rd, conv);
   };
   // parking record r: the iterate, -q, the iteration count and the slot
   auto park_store = [&](int r) {
@@ -311,15 +311,30 @@ __global__ void __launch_bounds__(CTA_LANES, 4) qp_solve_kernel(const float* __r
   const int nw = min(32, (int)blockDim.x - 32 * warp);
   const unsigned wmask = nw == 32 ? 0xffffffffu : (1u << nw) - 1u;  // this warp's threads
   int warps = (blockDim.x + 31) / 32;                                  // warps that hold running QPs
-  // warps that take wide groups: warp 0 when it is full and the parking area
-  // has room.  (Groups in every full warp, up to 18 QPs at m = 5, took
-  // 3.05 ms on the paper batch against 2.68 ms for warp 0 alone: the SMs
-  // turn issue-bound again.)
-  const int wide_warps = (blockDim.x >= 32 && GPB * S * L::PW >= L::QPW * L::WIDE_PER_QP) ? 1 : 0;
-  const bool wide_ok = cfg.eps > 0.f && wide_warps > 0;
-  int n_run;
+  const int wide_warps = blockDim.x / 32;  // the CTA's full warps take wide groups
+  // the running QPs into the parking area, in thread order (every thread)
+  auto compact = [&]() {
+    const unsigned bal = __ballot_sync(wmask, p >= 0);
+    if (wl == 0) wcount[warp] = __popc(bal);
+    __syncthreads();
+    if (p >= 0) {
+      int r = __popc(bal & ((1u << wl) - 1u));
+      for (int k = 0; k < warp; ++k) r += wcount[k];
+      park_store(r);
+    }
+    __syncthreads();
+  };
+  int n_run = __syncthreads_count(p >= 0);
 #pragma unroll 1
   for (;;) {
+    if (n_run <= wide_warps * L::QPW) break;  // the rest in the wide form
+    if ((n_run + 31) / 32 < warps) {
+      // repack: running QPs, in thread order, to threads 0 .. n_run - 1
+      compact();
+      p = -1;
+      if ((int)threadIdx.x < n_run) park_load(threadIdx.x);
+      warps = (n_run + 31) / 32;
+    }
     bool run = p >= 0;
     if (run) {
       const int g = p / S;
@@ -339,13 +354,13 @@ __global__ void __launch_bounds__(CTA_LANES, 4) qp_solve_kernel(const float* __r
       park_store(threadIdx.x);
       {
         const float* rec = park + threadIdx.x * L::PW;
-        if (CONE == CONE_SOC) admm_residuals_soc<M, true>(rec, rec + L::pW, rec + L::pM, Gg, cfg, rho, rp, rd, scale);
-        else admm_residuals<M, true>(rec, rec + L::pW, rec + L::pM, Gg, cfg, rho, rp, rd, scale);
+        if (CONE == CONE_SOC) admm_residuals_soc<M, ADAPT>(rec, rec + L::pW, rec + L::pM, Gg, cfg, rho, rp, rd, scale);
+        else admm_residuals<M, ADAPT>(rec, rec + L::pW, rec + L::pM, Gg, cfg, rho, rp, rd, scale);
       }
       park_load(threadIdx.x);
       const bool conv = cfg.eps > 0.f && rp <= cfg.eps && rd <= cfg.eps;
       if (conv || it >= cfg.iters) {
-        finish(p, rp, rd, conv);
+        finish_lane(p, rp, rd, conv);
         run = false;
       }
       // residual balancing (OSQP, Stellato et al. 2020, Sec. 5.2): each
@@ -356,7 +371,7 @@ __global__ void __launch_bounds__(CTA_LANES, 4) qp_solve_kernel(const float* __r
     n_run = __syncthreads_count(run);
     if (n_run == 0) break;
     if (adaptive) {
-      if (!__syncthreads_or(decide())) goto repack;  // no grasp of the CTA changed rho
+      if (!__syncthreads_or(decide())) continue;  // no grasp of the CTA changed rho
       const bool mine = p >= 0;
       if (mine) {  // re-express the iterate at the grasp's new rho, then park it (its registers go to the setup)
         const float* pg = per(p / S);
@@ -366,204 +381,121 @@ __global__ void __launch_bounds__(CTA_LANES, 4) qp_solve_kernel(const float* __r
       rebuild();
       if (mine) park_load(threadIdx.x);
     }
-  repack:
-    if (wide_ok && n_run <= wide_warps * L::QPW) {
-      // to the wide form: the running QPs parked in thread order (record r)
-      const unsigned bal = __ballot_sync(wmask, p >= 0);
-      if (wl == 0) wcount[warp] = __popc(bal);
-      __syncthreads();
-      if (p >= 0) {
-        int r = __popc(bal & ((1u << wl) - 1u));
-        for (int k = 0; k < warp; ++k) r += wcount[k];
-        park_store(r);
-      }
-      __syncthreads();
-      break;
-    }
-    if ((n_run + 31) / 32 < warps) {
-      // repack: running QPs, in thread order, to threads 0 .. n_run - 1
-      const unsigned bal = __ballot_sync(wmask, p >= 0);
-      if (wl == 0) wcount[warp] = __popc(bal);
-      __syncthreads();
-      if (p >= 0) {
-        int r = __popc(bal & ((1u << wl) - 1u));
-        for (int k = 0; k < warp; ++k) r += wcount[k];
-        park_store(r);
-      }
-      __syncthreads();
-      p = -1;
-      if ((int)threadIdx.x < n_run) park_load(threadIdx.x);
-      warps = (n_run + 31) / 32;
-    }
   }
-  if (n_run == 0) return;
-  // wide form (see above): group gi (QPW per wide warp) takes record gi,
-  // its lane ci the rows of contact ci and a dense copy of rows 3ci .. 3ci+2
-  // of the grasp's alpha K^-1 (in the parking area, after the records)
-  constexpr int WPC = L::WPC, NVP = L::NVP;
+  compact();
+  // wide form (see above): the n_run parked QPs over as few warps as hold
+  // them (record r on warp r mod ww), m lanes each
   const int ci = wl % M, gb = (wl / M) * M;  // contact; first lane of the group in the warp
-  const bool in_group = wl < L::QPW * M;     // lanes past the last whole group stay idle
-  const int gi = warp * L::QPW + (in_group ? wl / M : 0);
-  float wy[3] = {0.f, 0.f, 0.f}, ww[WPC], wmq[3] = {0.f, 0.f, 0.f}, wsum = 0.f;
-#pragma unroll
-  for (int k = 0; k < WPC; ++k) ww[k] = 0.f;
-  float* Kd = park;  // any valid address for an idle lane
+  const bool group_lane = wl < L::QPW * M;   // lanes past the last whole group stay idle
+  Wide<M, CONE> W;
+  W.clear();
   p = -1;
-  const bool wide_warp = warp < wide_warps;
-  if (wide_warp && in_group && gi < n_run) {
-    const float* rec = park + gi * L::PW;
-    it = reinterpret_cast<const int*>(rec)[L::pI];
-    p = reinterpret_cast<const int*>(rec)[L::pI + 1];
+  int ww = 0;  // warps that hold running QPs
+  auto spread = [&]() {
+    ww = (n_run + L::QPW - 1) / L::QPW;
+    const int r = ww * (wl / M) + warp;
+    p = -1;
+    if (warp < ww && group_lane && r < n_run) {
+      const float* rec = park + r * L::PW;
+      it = reinterpret_cast<const int*>(rec)[L::pI];
+      p = reinterpret_cast<const int*>(rec)[L::pI + 1];
 #pragma unroll
-    for (int r = 0; r < 3; ++r) {
-      wy[r] = rec[3 * ci + r];
-      wmq[r] = rec[L::pM + 3 * ci + r];
-    }
-#pragma unroll
-    for (int k = 0; k < WPC; ++k) ww[k] = rec[L::pW + WPC * ci + k];
-    wsum = rec[L::pW + NC - 1];
-    Kd = park + wide_warps * L::QPW * L::PW + gi * (NV * NVP) + 3 * ci * NVP;
-  }
-  // rows 3ci .. 3ci+2 of the grasp's alpha K^-1, dense (this lane's own rows)
-  auto copy_rows = [&]() {
-    const float* kg = kin(p / S);
-#pragma unroll
-    for (int r = 0; r < 3; ++r)
-#pragma unroll
-      for (int j = 0; j < NVP; ++j) {
-        const int a = min(3 * ci + r, j), b = max(3 * ci + r, j);
-        Kd[r * NVP + j] = j < NV ? kg[Admm<M>::tri(a, b)] : 0.f;
+      for (int k = 0; k < 3; ++k) {
+        W.y[k] = rec[3 * ci + k];
+        W.mq[k] = rec[L::pM + 3 * ci + k];
       }
+#pragma unroll
+      for (int k = 0; k < L::WPC; ++k) W.w[k] = rec[L::pW + L::WPC * ci + k];
+      W.wsum = rec[L::pW + NC - 1];
+      W.load_rows(kin(p / S), ci);
+    }
   };
-  if (p >= 0) copy_rows();
+  spread();
 #pragma unroll 1
   for (;;) {
     bool run = false;
-    if (wide_warp) {
+    if (warp < ww) {
       const bool mine = p >= 0;
       const int g = mine ? p / S : 0;
       const float rho = per(g)[L::oRho];
+      const float* Gg = per(g) + L::oG;
       // running QPs advance in lockstep rounds, so they share `it`
       const int chunk = __reduce_max_sync(0xffffffffu, mine ? min(check, cfg.iters - it) : 0);
-      const float al = cfg.alpha, bl = 1.0f - cfg.alpha;
 #pragma unroll 1
-      for (int k = 0; k < chunk; ++k) {
-        const float vsum = fmaf(2.f, fmaxf(wsum, cfg.gamma), -wsum);
-        float rhs3[3], pc3[3];
-        if (CONE == CONE_SOC) soc_contact_rhs(ww, vsum, wy, wmq, cfg, rho, rhs3, pc3);
-        else pyr_contact_rhs(ww, vsum, wy, wmq, cfg, rho, rhs3);
-        float ra[NV];
-#pragma unroll
-        for (int j = 0; j < NV; ++j) ra[j] = __shfl_sync(0xffffffffu, rhs3[j % 3], gb + j / 3);
-        float yt3[3];
-#pragma unroll
-        for (int r = 0; r < 3; ++r) {
-          const float4* row = reinterpret_cast<const float4*>(Kd + r * NVP);
-          float acc = 0.f;
-#pragma unroll
-          for (int j4 = 0; j4 < NVP / 4; ++j4) {
-            const float4 kv = row[j4];
-            if (4 * j4 + 0 < NV) acc = fmaf(kv.x, ra[4 * j4 + 0], acc);
-            if (4 * j4 + 1 < NV) acc = fmaf(kv.y, ra[4 * j4 + 1], acc);
-            if (4 * j4 + 2 < NV) acc = fmaf(kv.z, ra[4 * j4 + 2], acc);
-            if (4 * j4 + 3 < NV) acc = fmaf(kv.w, ra[4 * j4 + 3], acc);
-          }
-          yt3[r] = acc;
-        }
-        float sumn = 0.f;
-#pragma unroll
-        for (int i = 0; i < M; ++i) sumn += __shfl_sync(0xffffffffu, yt3[0], gb + i);
-        if (CONE == CONE_SOC) soc_contact_update(ww, pc3, yt3[0], yt3[1], yt3[2], cfg);
-        else pyr_contact_update(ww, yt3[0], yt3[1], yt3[2], cfg);
-        wsum = fmaf(-al, fmaxf(wsum, cfg.gamma), wsum + sumn);
-#pragma unroll
-        for (int r = 0; r < 3; ++r) wy[r] = fmaf(bl, wy[r], yt3[r]);
-      }
+      for (int k = 0; k < chunk; ++k) W.iterate(cfg, rho, gb);
       it += chunk;
-      // residuals, spread over the group: every lane gathers y and forms
-      // G y, then its contact's primal rows and dual components; the group
-      // takes the maxima (the one-lane function's values, bitwise)
-      float ya[NV];
-#pragma unroll
-      for (int j = 0; j < NV; ++j) ya[j] = __shfl_sync(0xffffffffu, wy[j % 3], gb + j / 3);
-      const float* Gg = per(g) + L::oG;
-      float sumn = 0.f, rp = 0.f, rd = 0.f, np = 0.f, nd = 0.f;
-#pragma unroll
-      for (int i = 0; i < M; ++i) sumn += ya[3 * i];
-      float at[3];
-      const float psum = fmaxf(wsum, cfg.gamma), dsum = wsum - psum;
-      if (CONE == CONE_SOC) {
-        float dl[4];
-        if (adaptive) soc_contact_primal<true>(ww, wy[0], wy[1], wy[2], cfg, rp, np, dl);
-        else soc_contact_primal<false>(ww, wy[0], wy[1], wy[2], cfg, rp, np, dl);
-        at[0] = fmaf(cfg.mu, dl[1], dl[0]) + dsum;
-        at[1] = dl[2];
-        at[2] = dl[3];
-      } else {
-        if (adaptive) pyr_contact_primal<true>(ww, wy[0], wy[1], wy[2], cfg, rp, np);
-        else pyr_contact_primal<false>(ww, wy[0], wy[1], wy[2], cfg, rp, np);
-        pyr_contact_atd(ww, dsum, cfg, at);
-      }
-      rp = fmaxf(rp, fabsf(sumn - psum));
-      float gy[6];
-      g_times<NV>(Gg, ya, gy);
-#pragma unroll
-      for (int q = 0; q < 3; ++q) {
-        if (adaptive) dual_component<NV, true>(Gg, 3 * ci + q, gy, wy[q], wmq[q], at[q], cfg, rho, rd, nd);
-        else dual_component<NV, false>(Gg, 3 * ci + q, gy, wy[q], wmq[q], at[q], cfg, rho, rd, nd);
-      }
-      float rpg = 0.f, rdg = 0.f, scale[2] = {0.f, 0.f};  // group maxima (scales: adaptive rho only)
-#pragma unroll
-      for (int i = 0; i < M; ++i) {
-        rpg = fmaxf(rpg, __shfl_sync(0xffffffffu, rp, gb + i));
-        rdg = fmaxf(rdg, __shfl_sync(0xffffffffu, rd, gb + i));
-      }
-      if (adaptive) {
-        np = fmaxf(np, fmaxf(fabsf(sumn), fabsf(psum)));
-#pragma unroll
-        for (int i = 0; i < M; ++i) {
-          scale[0] = fmaxf(scale[0], __shfl_sync(0xffffffffu, np, gb + i));
-          scale[1] = fmaxf(scale[1], __shfl_sync(0xffffffffu, nd, gb + i));
-        }
-      }
+      float rpg, rdg, scale[2] = {0.f, 0.f};  // scales: adaptive rho only
+      if (adaptive) W.template residuals<true>(Gg, cfg, rho, ci, gb, rpg, rdg, scale);
+      else W.template residuals<false>(Gg, cfg, rho, ci, gb, rpg, rdg, scale);
       const bool conv = rpg <= cfg.eps && rdg <= cfg.eps;
       const bool done = mine && (conv || it >= cfg.iters);
       if (__any_sync(0xffffffffu, done)) {
-        // the finished groups' state into their records; their lane 0 writes the results
-        float* rec = park + gi * L::PW;
+        // the finished groups' results: each lane its contact's rows, the
+        // group's first lane the sum row, Q and the status
+        float ya[NV];
+#pragma unroll
+        for (int j = 0; j < NV; ++j) ya[j] = __shfl_sync(0xffffffffu, W.y[j % 3], gb + j / 3);
         if (done) {
+          const size_t q = q0 + p;
 #pragma unroll
-          for (int r = 0; r < 3; ++r) rec[3 * ci + r] = wy[r];
+          for (int r = 0; r < 3; ++r) yio[q * NV + 3 * ci + r] = W.y[r];
 #pragma unroll
-          for (int k = 0; k < WPC; ++k) rec[L::pW + WPC * ci + k] = ww[k];
-          if (ci == 0) rec[L::pW + NC - 1] = wsum;
+          for (int k = 0; k < L::WPC; ++k) {
+            const float pr = CONE == CONE_SOC ? proj_row_soc<1>(W.w, k, cfg.gamma) : proj_row<1>(W.w[k], k, cfg.gamma);
+            zio[q * NC + L::WPC * ci + k] = pr;
+            lio[q * NC + L::WPC * ci + k] = rho * (W.w[k] - pr);
+          }
+          if (ci == 0) {
+            const float pr = fmaxf(W.wsum, cfg.gamma);
+            zio[q * NC + NC - 1] = pr;
+            lio[q * NC + NC - 1] = rho * (W.wsum - pr);
+            finish(p, ya, rpg, rdg, conv);
+          }
         }
-        __syncwarp();
-        if (done && ci == 0) {
-#pragma unroll
-          for (int a = 0; a < NV; ++a) y[a] = rec[a];
-#pragma unroll
-          for (int r = 0; r < NC; ++r) w[r] = rec[L::pW + r];
-          finish(p, rpg, rdg, conv);
-        }
-        __syncwarp();
       }
       run = mine && !done && ci == 0;
       if (adaptive && mine && ci == 0) per(g)[L::oVote + p % S] = done ? 0.f : rho_vote(rpg, rdg, scale);
       if (done) p = -1;
     }
-    if (__syncthreads_count(run) == 0) break;
+    n_run = __syncthreads_count(run);
+    if (n_run == 0) break;
     if (adaptive && __syncthreads_or(decide())) {
       // the wide lanes re-express their rows at the grasp's new rho; after the
-      // rebuild they refresh their dense rows of K^-1
+      // rebuild they load their rows of K^-1 again
       const bool moved = p >= 0 && per(p / S)[L::oRho] != per(p / S)[L::oRho + 1];
       if (moved) {
         const float ratio = per(p / S)[L::oRho + 1] / per(p / S)[L::oRho];
-        rescale_contact<CONE>(ww, ratio);
-        wsum = rescale_sum_row(wsum, ratio, cfg.gamma);
+        rescale_contact<CONE>(W.w, ratio);
+        W.wsum = rescale_sum_row(W.wsum, ratio, cfg.gamma);
       }
       rebuild();
-      if (moved) copy_rows();
+      if (p >= 0) W.load_rows(kin(p / S), ci);  // every group: the rows need not live across the rebuild
+    }
+    if ((n_run + L::QPW - 1) / L::QPW < ww) {
+      // fewer warps hold the rest: their state through the parking area, in
+      // thread order
+      const unsigned bal = __ballot_sync(wmask, p >= 0 && ci == 0);
+      if (wl == 0) wcount[warp] = __popc(bal);
+      __syncthreads();
+      if (p >= 0) {
+        int r = __popc(bal & ((1u << gb) - 1u));
+        for (int k = 0; k < warp; ++k) r += wcount[k];
+        float* rec = park + r * L::PW;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          rec[3 * ci + k] = W.y[k];
+          rec[L::pM + 3 * ci + k] = W.mq[k];
+        }
+#pragma unroll
+        for (int k = 0; k < L::WPC; ++k) rec[L::pW + L::WPC * ci + k] = W.w[k];
+        if (ci == 0) {
+          rec[L::pW + NC - 1] = W.wsum;
+          reinterpret_cast<int*>(rec)[L::pI] = it;
+          reinterpret_cast<int*>(rec)[L::pI + 1] = p;
+        }
+      }
+      __syncthreads();
+      spread();
     }
   }
 }
@@ -1273,6 +1205,17 @@ inline int pick_gpb(int s, int requested) {
   return requested > 0 ? std::min(requested, cap) : cap;
 }
 
+// Multiprocessors of the current device (152 on a GB300).
+inline int sm_count() {
+  int dev = 0, n = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1) {
+    (void)cudaGetLastError();
+    n = 152;
+  }
+  return n;
+}
+
 // Raises the kernel's dynamic shared-memory limit when needed, once per
 // device and size (so that launches recorded into a CUDA graph issue no
 // attribute calls after the first).
@@ -1342,17 +1285,25 @@ inline int run_qp(const float* G, int B, const float* T, int s, const AdmmCfg& c
                                                                     res);
     return launch_err("qp_exact_kernel launch");
   }
-  const int gpb = cfg.cone ? qp_gpb<M, CONE_SOC>(s) : qp_gpb<M, CONE_PYR>(s);
+  // A small batch runs in the wide form from its first iteration, one grasp
+  // a block, while that takes at most two warps a scheduler: up to there an
+  // iteration is latency (see Wide).  Larger batches start with one QP a lane.
+  constexpr int QPW = Wide<M, CONE_PYR>::QPW;
+  const int wide_warps = (s + QPW - 1) / QPW;
+  const bool wide = (long long)B * wide_warps <= 8LL * sm_count();
+  const int gpb = wide ? 1 : cfg.cone ? qp_gpb<M, CONE_SOC>(s) : qp_gpb<M, CONE_PYR>(s);
+  const int threads = wide ? 32 * wide_warps : gpb * s;
   const size_t bytes = cfg.cone ? LayQP<M, CONE_SOC>::bytes(gpb, s) : LayQP<M, CONE_PYR>::bytes(gpb, s);
-  if (cfg.cone) {
-    if (int r = ensure_smem(qp_solve_kernel<M, CONE_SOC>, bytes)) return r;
-    qp_solve_kernel<M, CONE_SOC><<<(B + gpb - 1) / gpb, gpb * s, bytes, st>>>(G, B, T, s, cfg, warm, y, z, lam, Q,
-                                                                              iters, status, res);
-  } else {
-    if (int r = ensure_smem(qp_solve_kernel<M, CONE_PYR>, bytes)) return r;
-    qp_solve_kernel<M, CONE_PYR><<<(B + gpb - 1) / gpb, gpb * s, bytes, st>>>(G, B, T, s, cfg, warm, y, z, lam, Q,
-                                                                              iters, status, res);
-    if (int r = launch_err("qp_solve_kernel launch")) return r;
+  const bool adapt = cfg.eps > 0.f && cfg.adapt;
+  auto go = [&](auto kernel) -> int {
+    if (int r = ensure_smem(kernel, bytes)) return r;
+    kernel<<<(B + gpb - 1) / gpb, threads, bytes, st>>>(G, B, T, s, gpb, cfg, warm, y, z, lam, Q, iters, status, res);
+    return launch_err("qp_solve_kernel launch");
+  };
+  if (cfg.cone) return adapt ? go(qp_solve_kernel<M, CONE_SOC, true>) : go(qp_solve_kernel<M, CONE_SOC, false>);
+  {
+    const int r = adapt ? go(qp_solve_kernel<M, CONE_PYR, true>) : go(qp_solve_kernel<M, CONE_PYR, false>);
+    if (r) return r;
     if (cfg.polish == 1 && cfg.eps_reg == 0.f) {
       const size_t n = (size_t)B * s;
       qp_polish_kernel<M><<<(unsigned)((n + 127) / 128), 128, 0, st>>>(G, B, T, s, cfg, y, Q, status);
@@ -1366,7 +1317,6 @@ inline int run_qp(const float* G, int B, const float* T, int s, const AdmmCfg& c
     }
     return BODEX_OK;
   }
-  return launch_err("qp_solve_kernel launch");
 }
 
 // Launchers, one translation unit each (fused_m*.cu, qp.cu, fused_multi.cu).

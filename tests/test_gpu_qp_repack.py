@@ -63,3 +63,21 @@ def test_qp_repacking_edge_shapes(B, s):
         one = bx.bodex_qp_solve_batch(G[b:b + 1].contiguous(), T, prm)
         for k in ("y", "z", "lam", "Q", "iters", "status"):
             assert torch.equal(full[k][b:b + 1], one[k]), (b, k)
+
+
+@pytest.mark.parametrize("m,cone", [(3, 0), (4, 0), (5, 0), (3, 1), (5, 1)])
+@pytest.mark.parametrize("s", [1, 7, 12])
+@pytest.mark.parametrize("adaptive", [0, 1])
+def test_small_batches_start_in_the_wide_form(m, cone, s, adaptive):
+    """A small batch gives every QP m lanes from its first iteration, a large
+    one starts with a lane each (here 1300 grasps, with their last block
+    partial): results are bitwise equal."""
+    T = cuda(I.wrench_set(12)[:s].copy())
+    p, n = I.random_contacts(13, m, seed=98 + m)
+    G = cuda(O.grasp_matrix(p, n).astype(np.float32))
+    prm = bx.qp_params(eps_abs=1e-5, max_iter=1500, check_every=10, adaptive_rho=adaptive, cone=cone)
+    small = bx.bodex_qp_solve_batch(G, T, prm)
+    large = bx.bodex_qp_solve_batch(G.repeat(100, 1, 1)[:1299].contiguous(), T, prm)
+    for k in ("y", "z", "lam", "Q", "iters", "status", "res"):
+        for first in (0, 13 * 50, 13 * 98):
+            assert torch.equal(large[k][first:first + 13], small[k]), (k, first)
