@@ -220,6 +220,62 @@ __device__ inline void fk_link(const HandDev& H, int i, const float* x, Tf& T, f
   }
 }
 
+// Forward kinematics with the work spread over a grasp's lanes, the same
+// operations as fk_link in two parts with a barrier between them.  Part 1:
+// every joint's rotation (rq: 9 words a joint) and the root frame (rt:
+// 12 words), one lane each; the root is
+// joint number n.  Part 2: row r of a frame product needs only row r of its
+// left factor, so three lanes a contact walk the chain, each with one row of
+// the frames, and form one component of the contact point (c) and of the
+// joints' axes and points (jw).  With one lane a contact, five chain links
+// of a 22-joint hand took 4300 cycles together with the query.
+__device__ __forceinline__ void fk_joint(const HandDev& H, int j, const float* x, float* rq, float* rt) {
+  if (j < H.n) {
+    const float a[3] = {H.axis[j][0], H.axis[j][1], H.axis[j][2]};
+    float R[9];
+    rodrigues(a, x[6 + j], R);
+#pragma unroll
+    for (int e = 0; e < 9; ++e) rq[9 * j + e] = R[e];
+  } else {
+    Tf T;
+    float om[3][3];
+    root_frame(x, T, om);
+    store_frame(T, rt);
+  }
+}
+
+__device__ __forceinline__ void fk_row(const HandDev& H, int i, int r, const float* rq, const float* rt, float* c,
+                                       float* jw, float* frames) {
+  float T[3] = {rt[3 * r], rt[3 * r + 1], rt[3 * r + 2]}, t = rt[9 + r];
+  if (frames) {
+    float* f = frames + 12 * H.n;
+    f[3 * r] = T[0], f[3 * r + 1] = T[1], f[3 * r + 2] = T[2], f[9 + r] = t;
+  }
+  const int L = H.chain_len[i];
+  for (int k = 0; k < L; ++k) {
+    const int j = H.chain[i][k];
+    const float4* off = reinterpret_cast<const float4*>(H.offset[j]);
+    const float4 o0 = off[0], o1 = off[1], o2 = off[2];
+    const float* q = rq + 9 * j;
+    const float b0 = fmaf(T[0], o0.x, fmaf(T[1], o1.x, T[2] * o2.x));
+    const float b1 = fmaf(T[0], o0.y, fmaf(T[1], o1.y, T[2] * o2.y));
+    const float b2 = fmaf(T[0], o0.z, fmaf(T[1], o1.z, T[2] * o2.z));
+    t = fmaf(T[0], o0.w, fmaf(T[1], o1.w, fmaf(T[2], o2.w, t)));
+    jw[6 * k + r] = fmaf(b0, H.axis[j][0], fmaf(b1, H.axis[j][1], b2 * H.axis[j][2]));
+    jw[6 * k + 3 + r] = t;
+    T[0] = fmaf(b0, q[0], fmaf(b1, q[3], b2 * q[6]));
+    T[1] = fmaf(b0, q[1], fmaf(b1, q[4], b2 * q[7]));
+    T[2] = fmaf(b0, q[2], fmaf(b1, q[5], b2 * q[8]));
+    t = fmaf(b0, 0.f, fmaf(b1, 0.f, fmaf(b2, 0.f, t)));
+    if (frames) {
+      float* f = frames + 12 * j;
+      f[3 * r] = T[0], f[3 * r + 1] = T[1], f[3 * r + 2] = T[2], f[9 + r] = t;
+    }
+  }
+  const float* cl = H.clocal[i];
+  c[r] = fmaf(T[0], cl[0], fmaf(T[1], cl[1], fmaf(T[2], cl[2], t)));
+}
+
 __device__ __forceinline__ void tf_point(const Tf& T, const float* p, float* c) {
   c[0] = fmaf(T.R[0], p[0], fmaf(T.R[1], p[1], fmaf(T.R[2], p[2], T.t[0])));
   c[1] = fmaf(T.R[3], p[0], fmaf(T.R[4], p[1], fmaf(T.R[5], p[2], T.t[1])));
@@ -516,7 +572,9 @@ __device__ __forceinline__ void load_u_row(const R* Us, int i, R (&u)[7]) {
 // are formed in unrolled rounds (the fused step, which repeats the set-up
 // every upper step; the QP kernels set up once and keep the loops, which
 // need fewer registers next to their repacking state).
-template <int M, typename R, bool UNROLL = false>
+// ENTRIES: K^-1 by single entries over the lanes instead of by column pairs,
+// for the wide fused step, whose grasps have up to 3m + 1 lanes or more.
+template <int M, typename R, bool UNROLL = false, bool ENTRIES = false>
 __device__ inline void setup_kinv_woodbury(bool active, int lane, int S, const float* G, float* scratch, float* Kinv,
                                            const AdmmCfg& c) {
   constexpr int NV = 3 * M;
@@ -600,7 +658,7 @@ __device__ inline void setup_kinv_woodbury(bool active, int lane, int S, const f
       for (int a = 0; a < 7; ++a) ild[a] = Us[a * 8 + 7];  // the U rows below write entries 0..6 only
     }
   } else {
-    if (active) factor();
+    if (active && (!ENTRIES || lane < NV)) factor();  // the lanes that form rows of U
   }
   if (active) {
     const R s2 = sqrt(R(2)), sr = sqrt(R(c.rho));
@@ -647,7 +705,26 @@ __device__ inline void setup_kinv_woodbury(bool active, int lane, int S, const f
   // with the grasp's other lanes: at each i they all read the same row of U,
   // one broadcast load, where spreading single entries over the lanes had
   // each lane read two rows of its own per entry.
-  if (active) {
+  if constexpr (ENTRIES) {
+    // entry e of the triangle folded into a rectangle of W columns: row r
+    // holds row r of the triangle and, in its first columns, row NV - r (odd
+    // NV) or NV - 1 - r (even NV)
+    constexpr int W = NV % 2 ? NV : NV + 1, OFF = NV % 2 ? 0 : 1;
+    if (active)
+      for (int e = lane; e < NV * (NV + 1) / 2; e += S) {
+        const int r = e / W, cc = e % W;
+        const bool own = cc >= r + OFF;
+        const int i = own ? r : NV - OFF - r, j = own ? cc - OFF : i + cc;
+        R ui[7], uj[7];
+        load_u_row(Us, i, ui);
+        load_u_row(Us, j, uj);
+        R acc = 0;
+#pragma unroll
+        for (int a = 0; a < 7; ++a) acc = fma_r(ui[a], uj[a], acc);
+        const R di = (i % 3 == 0) ? idn : idt;
+        Kinv[Admm<M>::tri(i, j)] = (float)(R(c.alpha) * ((i == j ? di : R(0)) - acc));
+      }
+  } else if (active) {
     for (int p = lane; p < (NV + 1) / 2; p += S) {
       const int j1 = p, j2 = NV - 1 - p;
       R u1[7], u2[7];
@@ -1790,7 +1867,7 @@ struct Wide {
 #pragma unroll
     for (int r = 0; r < 3; ++r)
 #pragma unroll
-      for (int j = 0; j < NV; ++j) K[r][j] = kin[Admm<M>::tri(min(3 * ci + r, j), max(3 * ci + r, j))];
+      for (int j = 0; j < NV; ++j) K[r][j] = lds32(kin + Admm<M>::tri(min(3 * ci + r, j), max(3 * ci + r, j)));
   }
   __device__ __forceinline__ void iterate(const AdmmCfg& c, float rho, int gb) {
     const float vsum = fmaf(2.f, fmaxf(wsum, c.gamma), -wsum);

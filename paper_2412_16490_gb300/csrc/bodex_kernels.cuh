@@ -113,11 +113,11 @@ __device__ __forceinline__ bool finite3(const float* v) {
 // Double precision when the host asks for it (solves that iterate to a
 // tight residual target), single precision otherwise; the branch is
 // uniform per launch.
-template <int M, bool UNROLL = false>
+template <int M, bool UNROLL = false, bool ENTRIES = false>
 __device__ inline void setup_kinv(bool active, int lane, int S, const float* Gs, float* scratch, float* Kinv,
                                   const AdmmCfg& cfg) {
-  if (cfg.fp64_setup) setup_kinv_woodbury<M, double>(active, lane, S, Gs, scratch, Kinv, cfg);
-  else setup_kinv_woodbury<M, float, UNROLL>(active, lane, S, Gs, scratch, Kinv, cfg);
+  if (cfg.fp64_setup) setup_kinv_woodbury<M, double, false, ENTRIES>(active, lane, S, Gs, scratch, Kinv, cfg);
+  else setup_kinv_woodbury<M, float, UNROLL, ENTRIES>(active, lane, S, Gs, scratch, Kinv, cfg);
 }
 
 // ============================================================================ kernel: batched QP
@@ -697,6 +697,84 @@ enum { MODE_EVAL = 0, MODE_STEP = 1, MODE_ADJOINT = 2 };
 constexpr int CONE_ANY = -1;
 constexpr int CONE_EXACT = 2;
 
+// dE/dc of contact `lane` through its kinematic chain: the translation, the
+// root rotations and the chain joints (axes and points jw of the forward
+// pass), into the contact's record cb.
+__device__ __forceinline__ void chain_adjoint(const HandDev& H, int lane, const float* xs, const float* c,
+                                              const float* jw, const float* dEdc, float* cb) {
+  cb[0] = dEdc[0];
+  cb[1] = dEdc[1];
+  cb[2] = dEdc[2];
+  // root rotations rx, ry, rz: axes through t
+  {
+    float s1, c1, s2, c2;
+    angle_sincos(xs[3], &s1, &c1);
+    angle_sincos(xs[4], &s2, &c2);
+    const float om[3][3] = {{1.f, 0.f, 0.f}, {0.f, c1, s1}, {s2, -s1 * c2, c1 * c2}};
+    const float rel[3] = {c[0] - xs[0], c[1] - xs[1], c[2] - xs[2]};
+    for (int k3 = 0; k3 < 3; ++k3) {
+      float v[3];
+      cross3(om[k3], rel, v);
+      cb[3 + k3] = dEdc[0] * v[0] + dEdc[1] * v[1] + dEdc[2] * v[2];
+    }
+  }
+  const int Lc = H.chain_len[lane];
+  for (int kk = 0; kk < Lc; ++kk) {
+    const float rel[3] = {c[0] - jw[6 * kk + 3], c[1] - jw[6 * kk + 4], c[2] - jw[6 * kk + 5]};
+    float v[3];
+    cross3(jw + 6 * kk, rel, v);
+    cb[6 + kk] = dEdc[0] * v[0] + dEdc[1] * v[1] + dEdc[2] * v[2];
+  }
+}
+
+// The gradient of grasp b from its contacts' records (fixed order over the
+// contacts), coordinates spread over S lanes; in MODE_STEP the Adam step and
+// the clamp follow.
+template <int M, int MODE>
+__device__ __forceinline__ void assemble_step(const FusedArgs& A, const HandDev& H, int b, int lane, int S, int step,
+                                              float lb1, float lb2, float* per) {
+  using L = Lay<M>;
+  float* xs = per + L::oX;
+  float* ams = per + L::oAM;
+  float* avs = per + L::oAV;
+  const int D = H.D;
+  const float* cb = per + L::oCB;
+  const int tstep = A.t0 + step + 1;
+  // bias corrections 1 - b^t as 1 - 2^(t log2 b): a function of t alone,
+  // so a run split over several launches gives the same values
+  const float c1 = 1.f - exp2f((float)tstep * lb1), c2 = 1.f - exp2f((float)tstep * lb2);
+  const float ic1 = 1.f / c1, ic2 = 1.f / c2;  // once per step, not per coordinate
+  for (int k = lane; k < D; k += S) {
+    float g = 0.f;
+    if (k < 6) {
+#pragma unroll
+      for (int i = 0; i < M; ++i) g += cb[i * (6 + MAXCHAIN) + k];
+    } else {
+      float v[M];  // every load before the sum: a contact that the joint does not move adds 0
+#pragma unroll
+      for (int i = 0; i < M; ++i) {
+        const int pos = H.jpos[i][k - 6];
+        const float e = cb[i * (6 + MAXCHAIN) + 6 + max(pos, 0)];
+        v[i] = pos >= 0 ? e : 0.f;
+      }
+#pragma unroll
+      for (int i = 0; i < M; ++i) g += v[i];
+    }
+    if (A.coll) g += per[L::oGC + k];
+    if (MODE != MODE_STEP) {
+      if (A.dEdx) A.dEdx[(size_t)b * D + k] = g;
+    } else {
+      const float mm = fmaf(A.b1, ams[k], (1.f - A.b1) * g);
+      const float vv = fmaf(A.b2, avs[k], (1.f - A.b2) * g * g);
+      ams[k] = mm;
+      avs[k] = vv;
+      const float lr = k < 3 ? A.lr_t : A.lr_r;
+      const float xn = xs[k] - __fdividef(lr * (mm * ic1), sqrtf(vv * ic2) + A.adam_eps);
+      xs[k] = fminf(fmaxf(xn, H.qmin[k]), H.qmax[k]);
+    }
+  }
+}
+
 template <int M, int MODE, int CONE = CONE_ANY, bool ADAPT = false>
 __device__ __forceinline__ void fused_cta(const FusedArgs& A, int cta, int GPB, float* smem) {
   using L = Lay<M>;
@@ -706,6 +784,11 @@ __device__ __forceinline__ void fused_cta(const FusedArgs& A, int cta, int GPB, 
   const int gl = threadIdx.x / S, lane = threadIdx.x % S;
   const int b = cta * GPB + gl;
   const bool active = (gl < GPB) && (b < A.B);
+  // with s < m lanes a grasp, a lane takes several contacts; the
+  // fixed-iteration step does without the loop, which cost it 0.8% (13.63
+  // against 13.51 ms for 4096 grasps x 200 steps): run_fused gives its s < m
+  // cases to the wide form
+  constexpr bool ONE_CONTACT = MODE == MODE_STEP && !ADAPT && (CONE == CONE_PYR || CONE == CONE_SOC);
   const HandDev& H = *reinterpret_cast<const HandDev*>(smem);
   float* kin = smem + L::HAND_WORDS + gl * L::KS;
   float* per = smem + L::HAND_WORDS + GPB * L::KS + gl * L::PER;
@@ -766,18 +849,18 @@ __device__ __forceinline__ void fused_cta(const FusedArgs& A, int cta, int GPB, 
   const float lb1 = log2f(A.b1), lb2 = log2f(A.b2);
   for (int step = 0; step < A.n_steps; ++step) {
     // ---- A1-A3: kinematics, nearest-point query, grasp matrix (lane = contact)
-    if (active && lane < M) {
+    if (int i = lane; active && i < M) do {
       float c[3];
-      fk_contact(H, lane, xs, c, per + L::oJW + lane * MAXCHAIN * 6,
+      fk_contact(H, i, xs, c, per + L::oJW + i * MAXCHAIN * 6,
                  (A.coll && A.cd.K > 0) ? per + L::oK : nullptr);  // link frames for the collision spheres
       const ContactGeo k = contact_geometry(A.obj, c);
-      store_ct(per + L::oCT + L::CTW * lane, k);
-      write_G_block(k, lane, NV, Gs);
+      store_ct(per + L::oCT + L::CTW * i, k);
+      write_G_block(k, i, NV, Gs);
       int st = 0;
       if (k.degenerate) st |= BODEX_ST_DEGENERATE_NORMAL;
       if (!finite3(k.p) || !finite3(k.n) || !isfinite(k.phi)) st |= BODEX_ST_NONFINITE;
       if (st) atomicOr(stat, st);
-    }
+    } while (!ONE_CONTACT && (i += S) < M);
     __syncthreads();
     // ---- constraint energies on the collision spheres (Sec. IV-B)
     if (A.coll)
@@ -971,12 +1054,12 @@ __device__ __forceinline__ void fused_cta(const FusedArgs& A, int cta, int GPB, 
     // shared dE/dG needs one more
     if (A.dfc) __syncthreads();
     // ---- A7 (part 2): through the contact geometry and the kinematic chain
-    if (active && lane < M) {
-      const ContactGeo k = load_ct(per + L::oCT + L::CTW * lane);
+    if (int i = lane; active && i < M) do {
+      const ContactGeo k = load_ct(per + L::oCT + L::CTW * i);
       float cols[18];
       if (A.dfc) {
         for (int r = 0; r < 6; ++r)
-          for (int cc = 0; cc < 3; ++cc) cols[r * 3 + cc] = per[L::oDG + r * NV + 3 * lane + cc];
+          for (int cc = 0; cc < 3; ++cc) cols[r * 3 + cc] = per[L::oDG + r * NV + 3 * i + cc];
       } else {
         // this contact's three columns of dE/dG = -2 w_Q sum_j r_j y_j^T,
         // each entry summing j in four partial sums (j mod 4, the tail
@@ -991,7 +1074,7 @@ __device__ __forceinline__ void fused_cta(const FusedArgs& A, int cta, int GPB, 
           const float4 r03 = *reinterpret_cast<const float4*>(ry + j * L::RYW);
           const float2 r45 = *reinterpret_cast<const float2*>(ry + j * L::RYW + 4);
           const float rv[6] = {r03.x, r03.y, r03.z, r03.w, r45.x, r45.y};
-          const float* yj = ry + j * L::RYW + 8 + 3 * lane;
+          const float* yj = ry + j * L::RYW + 8 + 3 * i;
           const float yv[3] = {yj[0], yj[1], yj[2]};
 #pragma unroll
           for (int r = 0; r < 6; ++r)
@@ -1011,66 +1094,11 @@ __device__ __forceinline__ void fused_cta(const FusedArgs& A, int cta, int GPB, 
       }
       float dEdc[3];
       contact_adjoint(k, cols, 2.f * A.w_d * (k.phi - H.alpha - A.delta), dEdc);
-      const float* jw = per + L::oJW + lane * MAXCHAIN * 6;  // frames from the forward pass
-      const float* c = k.c;
-      float* cb = per + L::oCB + lane * (6 + MAXCHAIN);
-      cb[0] = dEdc[0];
-      cb[1] = dEdc[1];
-      cb[2] = dEdc[2];
-      // root rotations rx, ry, rz: axes through t
-      {
-        float s1, c1, s2, c2;
-        angle_sincos(xs[3], &s1, &c1);
-        angle_sincos(xs[4], &s2, &c2);
-        const float om[3][3] = {{1.f, 0.f, 0.f}, {0.f, c1, s1}, {s2, -s1 * c2, c1 * c2}};
-        const float rel[3] = {c[0] - xs[0], c[1] - xs[1], c[2] - xs[2]};
-        for (int k3 = 0; k3 < 3; ++k3) {
-          float v[3];
-          cross3(om[k3], rel, v);
-          cb[3 + k3] = dEdc[0] * v[0] + dEdc[1] * v[1] + dEdc[2] * v[2];
-        }
-      }
-      const int Lc = H.chain_len[lane];
-      for (int kk = 0; kk < Lc; ++kk) {
-        const float rel[3] = {c[0] - jw[6 * kk + 3], c[1] - jw[6 * kk + 4], c[2] - jw[6 * kk + 5]};
-        float v[3];
-        cross3(jw + 6 * kk, rel, v);
-        cb[6 + kk] = dEdc[0] * v[0] + dEdc[1] * v[1] + dEdc[2] * v[2];
-      }
-    }
+      chain_adjoint(H, i, xs, k.c, per + L::oJW + i * MAXCHAIN * 6, dEdc, per + L::oCB + i * (6 + MAXCHAIN));
+    } while (!ONE_CONTACT && (i += S) < M);
     __syncthreads();
     // ---- gradient assembly (fixed order over contacts) and A8: Adam + clamp
-    if (active) {
-      const float* cb = per + L::oCB;
-      const int tstep = A.t0 + step + 1;
-      // bias corrections 1 - b^t as 1 - 2^(t log2 b): a function of t alone,
-      // so a run split over several launches gives the same values
-      const float c1 = 1.f - exp2f((float)tstep * lb1), c2 = 1.f - exp2f((float)tstep * lb2);
-      const float ic1 = 1.f / c1, ic2 = 1.f / c2;  // once per step, not per coordinate
-      for (int k = lane; k < D; k += S) {
-        float g = 0.f;
-        if (k < 6) {
-          for (int i = 0; i < M; ++i) g += cb[i * (6 + MAXCHAIN) + k];
-        } else {
-          for (int i = 0; i < M; ++i) {
-            const int pos = H.jpos[i][k - 6];
-            if (pos >= 0) g += cb[i * (6 + MAXCHAIN) + 6 + pos];
-          }
-        }
-        if (A.coll) g += per[L::oGC + k];
-        if (MODE != MODE_STEP) {
-          if (A.dEdx) A.dEdx[(size_t)b * D + k] = g;
-        } else {
-          const float mm = fmaf(A.b1, ams[k], (1.f - A.b1) * g);
-          const float vv = fmaf(A.b2, avs[k], (1.f - A.b2) * g * g);
-          ams[k] = mm;
-          avs[k] = vv;
-          const float lr = k < 3 ? A.lr_t : A.lr_r;
-          const float xn = xs[k] - __fdividef(lr * (mm * ic1), sqrtf(vv * ic2) + A.adam_eps);
-          xs[k] = fminf(fmaxf(xn, H.qmin[k]), H.qmax[k]);
-        }
-      }
-    }
+    if (active) assemble_step<M, MODE>(A, H, b, lane, S, step, lb1, lb2, per);
     __syncthreads();
   }
 
@@ -1108,6 +1136,357 @@ template <int M, int MODE, int CONE, bool ADAPT>
 __global__ void __launch_bounds__(CTA_LANES, 4) fused_kernel(FusedArgs A) {
   extern __shared__ __align__(16) float smem[];
   fused_cta<M, MODE, CONE, ADAPT>(A, blockIdx.x, A.gpb, smem);
+}
+
+// ============================================================================ kernel: fused evaluation / step, wide form
+// The fused step with m lanes per QP (Wide) instead of one, for fixed rho:
+// the CTA's GPB * s QPs lie one after another over its warps, 32 / m a warp,
+// and the lanes of a grasp, all threads of the CTA over GPB, share its set-up
+// phases.  Per lane the iterate is 13 words, so it stays in registers from
+// step to step.  Results are bitwise those of fused_cta.
+constexpr int WIDE_THREADS = 128;
+
+template <int M, int MODE, int CONE>
+__device__ __forceinline__ void fused_wide_cta(const FusedArgs& A, int cta, int GPB, float* smem) {
+  using L = Lay<M>;
+  using WQ = Wide<M, CONE>;
+  constexpr int NV = L::NV, WPC = WQ::WPC, QPW = WQ::QPW;
+  copy_hand_to_smem(A.hand, smem);
+  const HandDev& H = *reinterpret_cast<const HandDev*>(smem);
+  const int S = A.S, LN = blockDim.x / GPB;  // LN >= s m lanes per grasp
+  // A thread's two roles: lane `lane` of grasp gl in the set-up phases, and
+  // lane ci of the group (from lane gb of the warp) that holds wrench j of
+  // grasp gq.  Between the phases they live in two words: what follows from
+  // them is formed again in each phase (the compiler does not see that
+  // word() returns the same value), or some thirty pointers and indices
+  // stayed in registers across the ADMM loop and its K^-1 rows spilled (600
+  // cycles an iteration instead of 237).
+  auto word = [](int w) {
+    asm volatile("" : "+r"(w));
+    return w;
+  };
+  struct SetUp {
+    int lane, b;
+    bool active;
+    float *per, *kin;
+  };
+  struct Solve {
+    int ci, gb, j;
+    bool mine;
+    float *per, *kin;
+    size_t q;
+  };
+  const int w_set = (threadIdx.x / LN) << 16 | (threadIdx.x % LN);
+  int w_qp;
+  {
+    const int wl = threadIdx.x % 32, qi = (threadIdx.x / 32) * QPW + min(wl / M, QPW - 1), gq = min(qi / S, GPB - 1);
+    const bool mine = wl < QPW * M && qi < GPB * S && cta * GPB + gq < A.B;
+    w_qp = (mine ? 1 << 24 : 0) | gq << 16 | (qi % S) << 8 | (wl % M);
+  }
+  auto set_up = [&]() {
+    const int w = word(w_set), gl = w >> 16, g = min(gl, GPB - 1);
+    SetUp r;
+    r.lane = w & 0xffff;
+    r.b = cta * GPB + gl;
+    r.active = gl < GPB && r.b < A.B;
+    r.kin = smem + L::HAND_WORDS + g * L::KS;
+    r.per = smem + L::HAND_WORDS + GPB * L::KS + g * L::PER;
+    return r;
+  };
+  auto solve = [&]() {
+    const int w = word(w_qp), gq = (w >> 16) & 0xff;
+    Solve r;
+    r.ci = w & 0xff;
+    r.gb = ((threadIdx.x % 32) / M) * M;
+    r.j = (w >> 8) & 0xff;
+    r.mine = w >> 24;
+    r.kin = smem + L::HAND_WORDS + gq * L::KS;
+    r.per = smem + L::HAND_WORDS + GPB * L::KS + gq * L::PER;
+    r.q = (size_t)(cta * GPB + gq) * S + r.j;
+    return r;
+  };
+  const size_t NQ = (size_t)A.B * S;
+  __syncthreads();  // hand copied
+  const int D = H.D;
+  const AdmmCfg& cfg = A.cfg;
+  if (const SetUp u = set_up(); u.active) {
+    float* const per = u.per;
+    const int lane = u.lane, b = u.b;
+    const float* xsrc = (MODE == MODE_STEP) ? A.x_state : A.x_in;
+    for (int k = lane; k < D; k += LN) {
+      per[L::oX + k] = xsrc[(size_t)b * D + k];
+      if (MODE == MODE_STEP) {
+        per[L::oAM + k] = A.am[(size_t)b * D + k];
+        per[L::oAV + k] = A.av[(size_t)b * D + k];
+      }
+    }
+    if (lane == 0) {
+      reinterpret_cast<int*>(per + L::oSC)[1] = 0;  // status
+      per[L::oSC + 2] = 0.f;                        // max residual of the grasp's QPs at the last step
+    }
+  }
+  WQ W;
+  W.clear();
+  const bool warm = MODE == MODE_STEP || A.qy;
+  if (const Solve v = solve(); v.mine && warm) {
+    const int ci = v.ci;
+    const size_t q = v.q;
+#pragma unroll
+    for (int r = 0; r < 3; ++r) W.y[r] = A.qy[(3 * ci + r) * NQ + q];
+#pragma unroll
+    for (int k = 0; k < WPC; ++k) W.w[k] = A.qw[(WPC * ci + k) * NQ + q];
+    W.wsum = A.qw[WPC * M * NQ + q];
+  }
+  __syncthreads();
+
+#pragma unroll 1
+  for (int step = 0; step < A.n_steps; ++step) {
+    const bool last = step == A.n_steps - 1;
+    // ---- A1-A3: kinematics, nearest-point query, grasp matrix (lane = contact)
+    // (rotations and root frame in the records of the QP outputs, which are
+    // written after them)
+    static_assert(SMAX * L::RYW >= 9 * MAXJ + 12, "room for the joint rotations");
+    if (const SetUp u = set_up(); u.active)
+      for (int e = u.lane; e <= H.n; e += LN)
+        fk_joint(H, e, u.per + L::oX, u.per + L::oRY, u.per + L::oRY + 9 * MAXJ);
+    __syncthreads();
+    if (const SetUp u = set_up(); u.active)
+      for (int e = u.lane; e < 3 * M; e += LN)
+        fk_row(H, e / 3, e % 3, u.per + L::oRY, u.per + L::oRY + 9 * MAXJ, u.per + L::oCT + L::CTW * (e / 3),
+               u.per + L::oJW + (e / 3) * MAXCHAIN * 6,
+               (A.coll && A.cd.K > 0) ? u.per + L::oK : nullptr);  // link frames for the collision spheres
+    __syncthreads();
+    if (const SetUp u = set_up(); u.active && u.lane < M) {
+      float* const per = u.per;
+      const int lane = u.lane;
+      const float* rec = per + L::oCT + L::CTW * lane;
+      const float c[3] = {rec[0], rec[1], rec[2]};
+      const ContactGeo k = contact_geometry(A.obj, c);
+      store_ct(per + L::oCT + L::CTW * lane, k);
+      write_G_block(k, lane, NV, per + L::oG);
+      int st = 0;
+      if (k.degenerate) st |= BODEX_ST_DEGENERATE_NORMAL;
+      if (!finite3(k.p) || !finite3(k.n) || !isfinite(k.phi)) st |= BODEX_ST_NONFINITE;
+      if (st) atomicOr(reinterpret_cast<int*>(per + L::oSC + 1), st);
+    }
+    __syncthreads();
+    // ---- constraint energies: s lanes, as in fused_cta (the energy is summed lane by lane)
+    if (A.coll) {
+      const SetUp u = set_up();
+      float* const per = u.per;
+      collision_phase(u.active && u.lane < S, u.lane, S, H, A.cd, A.obj, per + L::oX, A.cp, per + L::oK, per + L::oJW,
+                      per + L::oRY, per + L::oRY + 3 * A.cd.K, per + L::oRY + 3 * A.cd.K + 6 * (H.n + 1),
+                      per + L::oGC, per + L::oGC + MAXD);
+    }
+    // ---- A4: K^-1 per grasp
+    {
+      const SetUp u = set_up();
+      setup_kinv<M, false, true>(u.active, u.lane, LN, u.per + L::oG, u.per + L::oK, u.kin, cfg);
+    }
+    // ---- A5: ADMM, one QP per m lanes
+    {
+      const Solve v = solve();
+      W.load_rows(v.kin, v.ci);
+      float t[6];
+#pragma unroll
+      for (int r = 0; r < 6; ++r) t[r] = __ldg(A.T + v.j * 6 + r);
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        float s = 0.f;
+#pragma unroll
+        for (int r = 0; r < 6; ++r) s = fmaf(v.per[L::oG + r * NV + 3 * v.ci + k], t[r], s);
+        W.mq[k] = 2.f * cfg.beta * s;
+      }
+    }
+    const int gb = ((threadIdx.x % 32) / M) * M;
+    float rp = 0.f, rd = 0.f;
+    bool conv = false;
+    if (cfg.eps > 0.f) {
+      // to a residual: a QP that reaches it keeps its iterate while the
+      // others of its warp go on
+      float ky[3], kw[WPC], ksum = 0.f, krp = 0.f, krd = 0.f;
+#pragma unroll 1
+      for (int it = 0; it < cfg.iters;) {
+        const int chunk = min(cfg.check, cfg.iters - it);
+#pragma unroll 1
+        for (int k = 0; k < chunk; ++k) W.iterate(cfg, cfg.rho, gb);
+        it += chunk;
+        const Solve v = solve();
+        W.template residuals<false>(v.per + L::oG, cfg, cfg.rho, v.ci, gb, rp, rd, nullptr);
+        if (!conv) {
+          krp = rp;
+          krd = rd;
+          ksum = W.wsum;
+#pragma unroll
+          for (int r = 0; r < 3; ++r) ky[r] = W.y[r];
+#pragma unroll
+          for (int k = 0; k < WPC; ++k) kw[k] = W.w[k];
+          conv = rp <= cfg.eps && rd <= cfg.eps;
+        }
+        if (__all_sync(0xffffffffu, conv || !v.mine)) break;
+      }
+      if (cfg.iters > 0) {
+        rp = krp;
+        rd = krd;
+        W.wsum = ksum;
+#pragma unroll
+        for (int r = 0; r < 3; ++r) W.y[r] = ky[r];
+#pragma unroll
+        for (int k = 0; k < WPC; ++k) W.w[k] = kw[k];
+      }
+    } else {
+#pragma unroll 1
+      for (int it = 0; it < cfg.iters; ++it) W.iterate(cfg, cfg.rho, gb);
+      if (last) {
+        const Solve v = solve();
+        W.template residuals<false>(v.per + L::oG, cfg, cfg.rho, v.ci, gb, rp, rd, nullptr);
+      }
+      conv = true;
+    }
+    {
+      // r = beta t - G y (row r by lane r of the group, the last rows by the
+      // first lanes), Q, the status; y and r for the adjoint
+      const Solve u = solve();
+      const int ci = u.ci, j = u.j;
+      const bool mine = u.mine;
+      float* const perq = u.per;
+      const float* const Gq = perq + L::oG;
+      float* const ry = perq + L::oRY + j * L::RYW;
+      float ya[NV], s[(6 + M - 1) / M], Q = 0.f;
+#pragma unroll
+      for (int a = 0; a < NV; ++a) ya[a] = __shfl_sync(0xffffffffu, W.y[a % 3], gb + a / 3);
+#pragma unroll
+      for (int k = 0; k < (6 + M - 1) / M; ++k) {
+        const int r = min(ci + k * M, 5);
+        float v = cfg.beta * __ldg(A.T + j * 6 + r);
+#pragma unroll
+        for (int a = 0; a < NV; ++a) v = fmaf(-Gq[r * NV + a], ya[a], v);
+        s[k] = v;
+        if (mine && ci + k * M < 6) ry[r] = v;
+      }
+#pragma unroll
+      for (int r = 0; r < 6; ++r) {
+        const float v = __shfl_sync(0xffffffffu, s[r / M], gb + r % M);
+        Q = fmaf(v, v, Q);
+      }
+#pragma unroll
+      for (int a = 0; a < NV; ++a) Q = fmaf(cfg.eps_reg * ya[a], ya[a], Q);  // regularised value when eps_reg > 0
+      if (mine) {
+#pragma unroll
+        for (int r = 0; r < 3; ++r) ry[8 + 3 * ci + r] = W.y[r];
+        if (ci == 0) {
+          perq[L::oQ + j] = Q;
+          int st = 0;
+          if (cfg.eps > 0.f && !conv) st |= BODEX_ST_NOT_CONVERGED;
+          if (!isfinite(Q)) st |= BODEX_ST_NONFINITE;
+          if (st) atomicOr(reinterpret_cast<int*>(perq + L::oSC + 1), st);
+          if (last) atomicMax(reinterpret_cast<int*>(perq + L::oSC + 2), __float_as_int(fmaxf(rp, rd)));
+        }
+      }
+    }
+    __syncthreads();
+    // ---- A6: energy (the last lane);  A7 (part 1): dE/dG = -2 w_Q sum_j r_j y_j^T,
+    // three columns of one row and contact a task, each entry summing j in
+    // four partial sums (j mod 4, the tail into the first)
+    if (const SetUp u = set_up(); u.active) {
+      float* const per = u.per;
+      for (int e = u.lane; e < 6 * M; e += LN) {
+        const int i = e / 6, r = e % 6;
+        const float* rec = per + L::oRY;
+        float s[3][4];
+#pragma unroll
+        for (int cc = 0; cc < 3; ++cc)
+#pragma unroll
+          for (int u = 0; u < 4; ++u) s[cc][u] = 0.f;
+        auto acc = [&](int jj, int u) {
+          const float rv = rec[jj * L::RYW + r];
+#pragma unroll
+          for (int cc = 0; cc < 3; ++cc) s[cc][u] = fmaf(rv, rec[jj * L::RYW + 8 + 3 * i + cc], s[cc][u]);
+        };
+        int jj = 0;
+        for (; jj + 3 < S; jj += 4) {
+          acc(jj, 0);
+          acc(jj + 1, 1);
+          acc(jj + 2, 2);
+          acc(jj + 3, 3);
+        }
+        for (; jj < S; ++jj) acc(jj, 0);
+#pragma unroll
+        for (int cc = 0; cc < 3; ++cc)
+          per[L::oDG + 18 * i + 3 * r + cc] = -2.f * A.w_q * ((s[cc][0] + s[cc][1]) + (s[cc][2] + s[cc][3]));
+      }
+      if (u.lane == LN - 1) {
+        float EQ = 0.f;
+        for (int k = 0; k < S; ++k) EQ += per[L::oQ + k];
+        float Ed = 0.f;
+        for (int i = 0; i < M; ++i) {
+          const float r = per[L::oCT + L::CTW * i + 9] - H.alpha - A.delta;
+          Ed = fmaf(r, r, Ed);
+        }
+        float Ec = 0.f;
+        if (A.coll)
+          for (int l = 0; l < S; ++l) Ec += per[L::oGC + MAXD + l];
+        per[L::oSC] = A.w_q * EQ + A.w_d * Ed + Ec;
+      }
+    }
+    __syncthreads();
+    // ---- A7 (part 2): through the contact geometry and the kinematic chain
+    if (const SetUp u = set_up(); u.active && u.lane < M) {
+      float* const per = u.per;
+      const int lane = u.lane;
+      const ContactGeo k = load_ct(per + L::oCT + L::CTW * lane);
+      float cols[18];
+#pragma unroll
+      for (int e = 0; e < 18; ++e) cols[e] = per[L::oDG + 18 * lane + e];
+      float dEdc[3];
+      contact_adjoint(k, cols, 2.f * A.w_d * (k.phi - H.alpha - A.delta), dEdc);
+      chain_adjoint(H, lane, per + L::oX, k.c, per + L::oJW + lane * MAXCHAIN * 6, dEdc, per + L::oCB + lane * (6 + MAXCHAIN));
+    }
+    __syncthreads();
+    // ---- gradient assembly and A8: Adam + clamp
+    if (const SetUp u = set_up(); u.active)
+      assemble_step<M, MODE>(A, H, u.b, u.lane, LN, step, log2f(A.b1), log2f(A.b2), u.per);
+    __syncthreads();
+  }
+
+  if (const SetUp u = set_up(); u.active) {
+    const float* const per = u.per;
+    const int lane = u.lane, b = u.b;
+    if (lane == 0) {
+      if (A.E) A.E[b] = per[L::oSC];
+      if (A.status) A.status[b] = __float_as_int(per[L::oSC + 1]);
+      if (A.res) A.res[b] = per[L::oSC + 2];
+    }
+    if (MODE == MODE_STEP)
+      for (int k = lane; k < D; k += LN) {
+        A.x_state[(size_t)b * D + k] = per[L::oX + k];
+        A.am[(size_t)b * D + k] = per[L::oAM + k];
+        A.av[(size_t)b * D + k] = per[L::oAV + k];
+      }
+  }
+  if (const Solve v = solve(); v.mine) {
+    const int ci = v.ci;
+    const size_t q = v.q;
+    if (warm) {
+#pragma unroll
+      for (int r = 0; r < 3; ++r) A.qy[(3 * ci + r) * NQ + q] = W.y[r];
+#pragma unroll
+      for (int k = 0; k < WPC; ++k) A.qw[(WPC * ci + k) * NQ + q] = W.w[k];
+      if (ci == 0) A.qw[WPC * M * NQ + q] = W.wsum;
+    }
+    if (MODE == MODE_EVAL) {
+      if (A.Qout && ci == 0) A.Qout[q] = v.per[L::oQ + v.j];
+      if (A.yout)
+#pragma unroll
+        for (int r = 0; r < 3; ++r) A.yout[q * NV + 3 * ci + r] = W.y[r];
+    }
+  }
+}
+
+template <int M, int MODE, int CONE>
+__global__ void __launch_bounds__(WIDE_THREADS, 4) fused_wide_kernel(FusedArgs A) {
+  extern __shared__ __align__(16) float smem[];
+  fused_wide_cta<M, MODE, CONE>(A, blockIdx.x, A.gpb, smem);
 }
 
 // ============================================================================ kernel: several jobs in one launch
@@ -1216,6 +1595,43 @@ inline int sm_count() {
   return n;
 }
 
+// Threads of a wide CTA with gpb grasps: 32 / m QPs a warp.
+template <int M>
+inline int wide_threads(int gpb, int s) {
+  constexpr int QPW = 32 / M;
+  return 32 * ((gpb * s + QPW - 1) / QPW);
+}
+
+// Grasps per CTA of the wide fused step: one while the batch takes at most
+// two warps a scheduler (the shortest steps), else the count that leaves the
+// fewest lanes idle, the smallest on ties.
+template <int M>
+inline int wide_tile(int s, int B, int sms) {
+  if ((long long)B * wide_threads<M>(1, s) <= 8LL * 32 * sms) return 1;
+  int best = 1;
+  for (int g = 2; wide_threads<M>(g, s) <= WIDE_THREADS && g <= gpb_for<M>(s); ++g)
+    if (wide_threads<M>(g, s) * best < wide_threads<M>(best, s) * g) best = g;
+  return best;
+}
+
+// Whether the fused step runs B grasps of s QPs in the wide form (bitwise the
+// same results).  The wide form's time grows with the QPs per SM; the
+// one-lane form's steps up with each block of 96 lanes that an SM holds.
+// Measured (50 steps of 50 iterations, one-lane -> wide, us), five contacts:
+// 40 QPs an SM 1552 -> 800, 81: 1555 -> 1435, 118: 2334 -> 2089, 162:
+// 2325 -> 2460; four: 118: 1705 -> 1292, 142: 1706 -> 1675, 162:
+// 1700 -> 1871; three: 63: 829 -> 704, 79: 836 -> 875, 103: 1243 -> 877, 162:
+// 1243 -> 1488.  Elliptic cone, whose chain is longer: five contacts 162:
+// 3518 -> 3263, 189: 3521 -> 3497, 237: 4081 -> 4495; four 237: 3027 -> 2595;
+// three 81: 1543 -> 1354, 162: 1826 -> 1859.
+template <int M>
+inline bool wide_pays(int s, int B, bool soc, int sms) {
+  const long long n = (long long)B * s;
+  if (soc) return n <= (M == 5 ? 176LL : M == 4 ? 224LL : 128LL) * sms;
+  if (M == 3) return n <= 64LL * sms || (n > 96LL * sms && n <= 112LL * sms);  // a second one-lane block costs more
+  return n <= 128LL * sms;
+}
+
 // Raises the kernel's dynamic shared-memory limit when needed, once per
 // device and size (so that launches recorded into a CUDA graph issue no
 // attribute calls after the first).
@@ -1247,14 +1663,22 @@ inline int ensure_smem(K kernel, size_t bytes) {
 
 template <int M>
 inline int run_fused(int mode, const FusedArgs& A0, cudaStream_t st) {
+  if (A0.B == 0) return BODEX_OK;
   FusedArgs A = A0;
-  A.gpb = pick_gpb<M>(A.S, A0.gpb);
-  const int gpb = A.gpb;
-  const size_t bytes = Lay<M>::bytes(gpb);
-  const dim3 grid((A.B + gpb - 1) / gpb), block(gpb * A.S);
-  if (A.B == 0) return BODEX_OK;
   const bool soc = A.cfg.cone != 0;
   const bool adapt = A.cfg.eps > 0.f && A.cfg.adapt;
+  // the wide form: ADMM at a fixed rho, where it pays and no tile is asked
+  // for, and fewer wrenches than contacts (which the one-lane step does not take)
+  bool wide = mode != MODE_ADJOINT && A.cfg.solver != BODEX_QP_EXACT && !adapt && !A.dfc;
+  if (wide) {
+    const int sms = sm_count();
+    wide = A.S < M || (A0.gpb <= 0 && wide_pays<M>(A.S, A.B, soc, sms));
+    if (wide) A.gpb = wide_tile<M>(A.S, A.B, sms);
+  }
+  if (!wide) A.gpb = pick_gpb<M>(A.S, A0.gpb);
+  const int gpb = A.gpb;
+  const size_t bytes = Lay<M>::bytes(gpb);
+  const dim3 grid((A.B + gpb - 1) / gpb), block(wide ? wide_threads<M>(gpb, A.S) : gpb * A.S);
   auto go = [&](auto kernel) -> int {
     if (int r = ensure_smem(kernel, bytes)) return r;
     kernel<<<grid, block, bytes, st>>>(A);
@@ -1262,6 +1686,10 @@ inline int run_fused(int mode, const FusedArgs& A0, cudaStream_t st) {
   };
   int r;
   if (mode == MODE_ADJOINT) r = go(fused_kernel<M, MODE_ADJOINT, CONE_PYR, false>);  // no lower-level solve
+  else if (wide && mode == MODE_STEP)
+    r = soc ? go(fused_wide_kernel<M, MODE_STEP, CONE_SOC>) : go(fused_wide_kernel<M, MODE_STEP, CONE_PYR>);
+  else if (wide)
+    r = soc ? go(fused_wide_kernel<M, MODE_EVAL, CONE_SOC>) : go(fused_wide_kernel<M, MODE_EVAL, CONE_PYR>);
   else if (A.cfg.solver == BODEX_QP_EXACT)
     r = mode == MODE_STEP ? go(fused_kernel<M, MODE_STEP, CONE_EXACT, false>) : go(fused_kernel<M, MODE_EVAL, CONE_EXACT, false>);
   else if (mode == MODE_STEP)
