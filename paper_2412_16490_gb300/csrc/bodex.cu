@@ -157,7 +157,10 @@ __global__ void __launch_bounds__(FkTile<M>::THREADS) fk_contacts_kernel(const H
 // the final one.  One warp per grasp and RF_GPB warps a block, with no block
 // barrier between steps: lanes 0..m-1 own a contact's kinematics and adjoint,
 // all 32 lanes share each fingertip's samples (the queries are most of the
-// work: 160 a grasp and step), the gradient assembly and Adam.  With eight
+// work: 160 a grasp and step), the gradient assembly and Adam; the chains are
+// walked by three lanes a contact, one row of the frames each, and the lowest
+// sample found by two warp reductions (4096 grasps x 100 steps: 1.50 -> 1.37
+// ms together).  With eight
 // lanes a grasp and each contact's samples walked by one of them, a step of
 // 4096 grasps was bound by the latency of 32 queries in a row on 6.7 warps an
 // SM.
@@ -198,17 +201,15 @@ __device__ __forceinline__ int lowest_sample(const Tf& T, const float* __restric
       kbest = k;
     }
   }
-#pragma unroll
-  for (int off = 16; off >= 1; off >>= 1) {
-    const float b2 = __shfl_xor_sync(0xffffffffu, best, off);
-    const int k2 = __shfl_xor_sync(0xffffffffu, kbest, off);
-    if (b2 < best || (b2 == best && k2 < kbest)) {
-      best = b2;
-      kbest = k2;
-    }
-  }
-  phi = best;
-  return best < INFINITY ? kbest : 0;
+  // two warp reductions (five shuffles and compares of a pair each before):
+  // the smallest value as an integer of the same order, then the lowest index
+  // that has it; adding 0 makes the two zeros one
+  const int v = __float_as_int(best + 0.f);
+  const unsigned key = (unsigned)(v ^ ((v >> 31) | (int)0x80000000));
+  const unsigned lo = __reduce_min_sync(0xffffffffu, key);
+  kbest = __reduce_min_sync(0xffffffffu, key == lo ? kbest : 0x7fffffff);
+  phi = __int_as_float((lo & 0x80000000u) ? (int)(lo ^ 0x80000000u) : (int)~lo);
+  return phi < INFINITY ? kbest : 0;
 }
 
 // A link frame in shared memory, 12 words.
@@ -224,7 +225,8 @@ template <int M>
 __global__ void __launch_bounds__(32 * RF_GPB) refine_kernel(RefineArgs A) {
   constexpr int HW = Lay<M>::HAND_WORDS;
   constexpr int CBW = 6 + MAXCHAIN;
-  constexpr int PER = align4(3 * MAXD + M * CBW + M * MAXCHAIN * 6 + M * 12 + M + 4);
+  constexpr int oRQ = 3 * MAXD + M * CBW + M * MAXCHAIN * 6 + M * 12 + M + 1;  // joint rotations and the root frame
+  constexpr int PER = align4(oRQ + 9 * MAXJ + 12 + 4);
   __shared__ __align__(16) float smem[HW + RF_GPB * PER];
   copy_hand_to_smem(A.hand, smem);
   const int gl = threadIdx.x / 32, lane = threadIdx.x % 32;
@@ -252,11 +254,11 @@ __global__ void __launch_bounds__(32 * RF_GPB) refine_kernel(RefineArgs A) {
   int kbest = 0;
   for (int step = 0; step < A.n_steps; ++step) {
     const float* jw = jwall + (lane < M ? lane : 0) * MAXCHAIN * 6;
-    if (lane < M) {
-      Tf T;
-      fk_link(H, lane, xs, T, jwall + lane * MAXCHAIN * 6);
-      store_frame(T, frames + 12 * lane);
-    }
+    for (int e = lane; e <= H.n; e += 32) fk_joint(H, e, xs, per + oRQ, per + oRQ + 9 * MAXJ);
+    __syncwarp();
+    if (lane < 3 * M)
+      fk_row(H, lane / 3, lane % 3, per + oRQ, per + oRQ + 9 * MAXJ, jwall + (lane / 3) * MAXCHAIN * 6, nullptr,
+             frames + 12 * (lane / 3), nullptr);
     __syncwarp();
 #pragma unroll
     for (int i = 0; i < M; ++i) {
@@ -286,27 +288,7 @@ __global__ void __launch_bounds__(32 * RF_GPB) refine_kernel(RefineArgs A) {
       Ei[lane] = e;
       if (k.degenerate) atomicOr(stat, BODEX_ST_DEGENERATE_NORMAL);
       if (!isfinite(e)) atomicOr(stat, BODEX_ST_NONFINITE);
-      float* c = cb + lane * CBW;
-      c[0] = dEdc[0];
-      c[1] = dEdc[1];
-      c[2] = dEdc[2];
-      float s1, c1, s2, c2;
-      angle_sincos(xs[3], &s1, &c1);
-      angle_sincos(xs[4], &s2, &c2);
-      const float om[3][3] = {{1.f, 0.f, 0.f}, {0.f, c1, s1}, {s2, -s1 * c2, c1 * c2}};
-      const float rel[3] = {cf[0] - xs[0], cf[1] - xs[1], cf[2] - xs[2]};
-      for (int k3 = 0; k3 < 3; ++k3) {
-        float v[3];
-        cross3(om[k3], rel, v);
-        c[3 + k3] = dEdc[0] * v[0] + dEdc[1] * v[1] + dEdc[2] * v[2];
-      }
-      const int Lc = H.chain_len[lane];
-      for (int kk = 0; kk < Lc; ++kk) {
-        const float r2[3] = {cf[0] - jw[6 * kk + 3], cf[1] - jw[6 * kk + 4], cf[2] - jw[6 * kk + 5]};
-        float v[3];
-        cross3(jw + 6 * kk, r2, v);
-        c[6 + kk] = dEdc[0] * v[0] + dEdc[1] * v[1] + dEdc[2] * v[2];
-      }
+      chain_adjoint(H, lane, xs, cf, jw, dEdc, cb + lane * CBW);
     }
     __syncwarp();
     {
@@ -320,12 +302,18 @@ __global__ void __launch_bounds__(32 * RF_GPB) refine_kernel(RefineArgs A) {
       for (int k = lane; k < D; k += 32) {
         float g = 0.f;
         if (k < 6) {
+#pragma unroll
           for (int i = 0; i < M; ++i) g += cb[i * CBW + k];
         } else {
+          float v[M];  // every load before the sum: a contact that the joint does not move adds 0
+#pragma unroll
           for (int i = 0; i < M; ++i) {
             const int pos = H.jpos[i][k - 6];
-            if (pos >= 0) g += cb[i * CBW + 6 + pos];
+            const float e = cb[i * CBW + 6 + max(pos, 0)];
+            v[i] = pos >= 0 ? e : 0.f;
           }
+#pragma unroll
+          for (int i = 0; i < M; ++i) g += v[i];
         }
         const float mm = fmaf(A.b1, ams[k], (1.f - A.b1) * g);
         const float vv = fmaf(A.b2, avs[k], (1.f - A.b2) * g * g);
@@ -370,7 +358,8 @@ struct MetricsArgs {
 template <int M>
 __global__ void __launch_bounds__(32 * RF_GPB) metrics_kernel(MetricsArgs A) {
   constexpr int HW = Lay<M>::HAND_WORDS;
-  constexpr int PER = align4(MAXD) + 12 * M;
+  constexpr int oRQ = align4(MAXD) + 12 * M;  // joint rotations and the root frame
+  constexpr int PER = oRQ + 9 * MAXJ + 12;
   __shared__ __align__(16) float smem[HW + RF_GPB * PER];
   copy_hand_to_smem(A.hand, smem);
   const int gl = threadIdx.x / 32, lane = threadIdx.x % 32;
@@ -383,11 +372,10 @@ __global__ void __launch_bounds__(32 * RF_GPB) metrics_kernel(MetricsArgs A) {
   const int D = H.D, S = A.tips ? H.S : 0;
   for (int k = lane; k < D; k += 32) xs[k] = A.x[(size_t)b * D + k];
   __syncwarp();
-  if (lane < M) {
-    Tf T;
-    fk_link(H, lane, xs, T, nullptr);
-    store_frame(T, frames + 12 * lane);
-  }
+  for (int e = lane; e <= H.n; e += 32) fk_joint(H, e, xs, xs + oRQ, xs + oRQ + 9 * MAXJ);
+  __syncwarp();
+  if (lane < 3 * M)
+    fk_row(H, lane / 3, lane % 3, xs + oRQ, xs + oRQ + 9 * MAXJ, nullptr, nullptr, frames + 12 * (lane / 3), nullptr);
   __syncwarp();
   float d = 0.f;
   if (S > 0) {

@@ -227,8 +227,8 @@ __device__ inline void fk_link(const HandDev& H, int i, const float* x, Tf& T, f
 // joint number n.  Part 2: row r of a frame product needs only row r of its
 // left factor, so three lanes a contact walk the chain, each with one row of
 // the frames, and form one component of the contact point (c) and of the
-// joints' axes and points (jw).  With one lane a contact, five chain links
-// of a 22-joint hand took 4300 cycles together with the query.
+// joints' axes and points (jw).  c, jw, frames (every chain link at 12 j, the
+// root at 12 n) and link (contact i's own link frame) may be null.
 __device__ __forceinline__ void fk_joint(const HandDev& H, int j, const float* x, float* rq, float* rt) {
   if (j < H.n) {
     const float a[3] = {H.axis[j][0], H.axis[j][1], H.axis[j][2]};
@@ -244,8 +244,8 @@ __device__ __forceinline__ void fk_joint(const HandDev& H, int j, const float* x
   }
 }
 
-__device__ __forceinline__ void fk_row(const HandDev& H, int i, int r, const float* rq, const float* rt, float* c,
-                                       float* jw, float* frames) {
+__device__ __forceinline__ void fk_row(const HandDev& H, int i, int r, const float* rq, const float* rt, float* jw,
+                                       float* c, float* link, float* frames) {
   float T[3] = {rt[3 * r], rt[3 * r + 1], rt[3 * r + 2]}, t = rt[9 + r];
   if (frames) {
     float* f = frames + 12 * H.n;
@@ -261,8 +261,10 @@ __device__ __forceinline__ void fk_row(const HandDev& H, int i, int r, const flo
     const float b1 = fmaf(T[0], o0.y, fmaf(T[1], o1.y, T[2] * o2.y));
     const float b2 = fmaf(T[0], o0.z, fmaf(T[1], o1.z, T[2] * o2.z));
     t = fmaf(T[0], o0.w, fmaf(T[1], o1.w, fmaf(T[2], o2.w, t)));
-    jw[6 * k + r] = fmaf(b0, H.axis[j][0], fmaf(b1, H.axis[j][1], b2 * H.axis[j][2]));
-    jw[6 * k + 3 + r] = t;
+    if (jw) {
+      jw[6 * k + r] = fmaf(b0, H.axis[j][0], fmaf(b1, H.axis[j][1], b2 * H.axis[j][2]));
+      jw[6 * k + 3 + r] = t;
+    }
     T[0] = fmaf(b0, q[0], fmaf(b1, q[3], b2 * q[6]));
     T[1] = fmaf(b0, q[1], fmaf(b1, q[4], b2 * q[7]));
     T[2] = fmaf(b0, q[2], fmaf(b1, q[5], b2 * q[8]));
@@ -272,8 +274,11 @@ __device__ __forceinline__ void fk_row(const HandDev& H, int i, int r, const flo
       f[3 * r] = T[0], f[3 * r + 1] = T[1], f[3 * r + 2] = T[2], f[9 + r] = t;
     }
   }
-  const float* cl = H.clocal[i];
-  c[r] = fmaf(T[0], cl[0], fmaf(T[1], cl[1], fmaf(T[2], cl[2], t)));
+  if (link) link[3 * r] = T[0], link[3 * r + 1] = T[1], link[3 * r + 2] = T[2], link[9 + r] = t;
+  if (c) {
+    const float* cl = H.clocal[i];
+    c[r] = fmaf(T[0], cl[0], fmaf(T[1], cl[1], fmaf(T[2], cl[2], t)));
+  }
 }
 
 __device__ __forceinline__ void tf_point(const Tf& T, const float* p, float* c) {

@@ -1252,8 +1252,8 @@ __device__ __forceinline__ void fused_wide_cta(const FusedArgs& A, int cta, int 
     __syncthreads();
     if (const SetUp u = set_up(); u.active)
       for (int e = u.lane; e < 3 * M; e += LN)
-        fk_row(H, e / 3, e % 3, u.per + L::oRY, u.per + L::oRY + 9 * MAXJ, u.per + L::oCT + L::CTW * (e / 3),
-               u.per + L::oJW + (e / 3) * MAXCHAIN * 6,
+        fk_row(H, e / 3, e % 3, u.per + L::oRY, u.per + L::oRY + 9 * MAXJ, u.per + L::oJW + (e / 3) * MAXCHAIN * 6,
+               u.per + L::oCT + L::CTW * (e / 3), nullptr,
                (A.coll && A.cd.K > 0) ? u.per + L::oK : nullptr);  // link frames for the collision spheres
     __syncthreads();
     if (const SetUp u = set_up(); u.active && u.lane < M) {
