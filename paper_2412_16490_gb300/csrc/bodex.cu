@@ -1002,6 +1002,16 @@ int bodex_step_multi(const bodex_job* jobs, int n_jobs, const bodex_step_params*
   std::memset(MA, 0, sizeof(MultiArgs));
   size_t bytes = 0;
   int total = 0, nj = 0;
+  // the wide form for all jobs or none: ADMM at a fixed rho, no tile or
+  // pulling asked for, and few enough QPs for it to pay (wide_limit)
+  const bool exact = params->qp.solver == BODEX_QP_EXACT;
+  const bool adapt = !exact && params->qp.eps_abs > 0.f && params->qp.adaptive_rho;
+  const bool soc = params->qp.cone != BODEX_CONE_PYRAMID;
+  bool wide = !exact && !adapt && params->energy.kind != BODEX_ENERGY_DFC && params->grasps_per_cta <= 0 && !params->work_pulling;
+  int threads = 0;
+  size_t wide_bytes = 0;
+  double wide_share = 0.0;  // of the QPs per SM up to which the wide form pays
+  const int sms = wide ? sm_count() : 1;
   int take[BODEX_MAX_JOBS], tiles[BODEX_MAX_JOBS];
   double cost[BODEX_MAX_JOBS];
   for (int j = 0; j < n_jobs; ++j) {
@@ -1041,15 +1051,28 @@ int bodex_step_multi(const bodex_job* jobs, int n_jobs, const bodex_step_params*
     A.status = J.status;
     A.res = S->res;
     MA->m[nj] = m;
+    switch (m) {
+      case 3: threads = std::max(threads, wide_threads<3>(1, J.s)); wide_bytes = std::max(wide_bytes, Lay<3>::bytes(1)); break;
+      case 4: threads = std::max(threads, wide_threads<4>(1, J.s)); wide_bytes = std::max(wide_bytes, Lay<4>::bytes(1)); break;
+      default: threads = std::max(threads, wide_threads<5>(1, J.s)); wide_bytes = std::max(wide_bytes, Lay<5>::bytes(1)); break;
+    }
+    wide_share += (double)S->B * J.s / ((double)wide_limit(m, soc) * sms);
     tiles[nj] = (S->B + gpb - 1) / gpb;
     // cost of one tile: steps x wrenches x (ADMM work per iteration, 26 m + 9 m^2 + ...,
     // taken as m^2; or m for the exact solve, whose oracle is linear in m)
-    const bool ex = params->qp.solver == BODEX_QP_EXACT;
-    cost[nj] = (double)J.n_steps * J.s * (ex ? m : m * m);
+    cost[nj] = (double)J.n_steps * J.s * (exact ? m : m * m);
     total += tiles[nj];
     bytes = std::max(bytes, b);
     take[nj] = j;
     ++nj;
+  }
+  wide = wide && wide_share <= 1.0;
+  if (wide) {
+    total = 0;
+    for (int k = 0; k < nj; ++k) {
+      MA->job[k].gpb = 1;
+      total += tiles[k] = MA->job[k].B;
+    }
   }
   MA->n_jobs = nj;
   MA->total = total;
@@ -1079,9 +1102,7 @@ int bodex_step_multi(const bodex_job* jobs, int n_jobs, const bodex_step_params*
         return cuda_fail(e, "cudaMemsetAsync(work counter)");
       }
     }
-    const bool exact = params->qp.solver == BODEX_QP_EXACT;
-    const bool adapt = !exact && params->qp.eps_abs > 0.f && params->qp.adaptive_rho;
-    r = launch_multi(adapt, exact, pull, *MA, bytes, st);
+    r = wide ? launch_multi_wide(soc, *MA, threads, wide_bytes, st) : launch_multi(adapt, exact, pull, *MA, bytes, st);
     if (r == BODEX_OK)
       for (int k = 0; k < nj; ++k) jobs[take[k]].state->t += jobs[take[k]].n_steps;
   }

@@ -1534,6 +1534,27 @@ __device__ __forceinline__ void multi_item(const MultiArgs& A, int w, float* sme
   }
 }
 
+// The same in the wide form (fixed rho, no pulling): every job's tile is one
+// grasp, blocks as wide as the widest job needs; a warp that a job leaves
+// without QPs still shares its set-up phases.  Taken when the jobs' shares of
+// wide_limit add up to at most 1: six jobs of three hands, 12 wrenches, 50
+// steps of 50 iterations take 912 us instead of 1772 with 200 grasps
+// together, 1321 (1873) with 900, 2396 (2553) with 1600; with 2000 the
+// one-lane form is ahead, 2586 against 2691.
+template <int CONE>
+__global__ void __launch_bounds__(WIDE_THREADS, 4) multi_wide_kernel(const __grid_constant__ MultiArgs A) {
+  extern __shared__ __align__(16) float smem[];
+  int k = 0;
+  while (k + 1 < A.n_jobs && (int)blockIdx.x >= A.order_begin[k + 1]) ++k;
+  const int j = A.order_job[k], cta = (int)blockIdx.x - A.order_begin[k];
+  const FusedArgs& J = A.job[j];
+  switch (A.m[j]) {
+    case 3: fused_wide_cta<3, MODE_STEP, CONE>(J, cta, 1, smem); break;
+    case 4: fused_wide_cta<4, MODE_STEP, CONE>(J, cta, 1, smem); break;
+    default: fused_wide_cta<5, MODE_STEP, CONE>(J, cta, 1, smem); break;
+  }
+}
+
 template <bool ADAPT, bool EXACT = false, bool PULL = false>
 __global__ void __launch_bounds__(CTA_LANES, 4) multi_kernel(const __grid_constant__ MultiArgs A) {
   extern __shared__ __align__(16) float smem[];
@@ -1624,12 +1645,15 @@ inline int wide_tile(int s, int B, int sms) {
 // 1243 -> 1488.  Elliptic cone, whose chain is longer: five contacts 162:
 // 3518 -> 3263, 189: 3521 -> 3497, 237: 4081 -> 4495; four 237: 3027 -> 2595;
 // three 81: 1543 -> 1354, 162: 1826 -> 1859.
+inline int wide_limit(int m, bool soc) {  // in QPs per SM
+  if (soc) return m == 5 ? 176 : m == 4 ? 224 : 128;
+  return m == 3 ? 64 : 128;
+}
 template <int M>
 inline bool wide_pays(int s, int B, bool soc, int sms) {
   const long long n = (long long)B * s;
-  if (soc) return n <= (M == 5 ? 176LL : M == 4 ? 224LL : 128LL) * sms;
-  if (M == 3) return n <= 64LL * sms || (n > 96LL * sms && n <= 112LL * sms);  // a second one-lane block costs more
-  return n <= 128LL * sms;
+  if (M == 3 && !soc && n > 96LL * sms && n <= 112LL * sms) return true;  // a second one-lane block costs more
+  return n <= (long long)wide_limit(M, soc) * sms;
 }
 
 // Raises the kernel's dynamic shared-memory limit when needed, once per
@@ -1754,3 +1778,4 @@ int launch_fused_m5(int mode, const FusedArgs& A, cudaStream_t st);
 int launch_qp(int m, const float* G, int B, const float* T, int s, const AdmmCfg& cfg, int warm, float* y, float* z,
               float* lam, float* Q, int32_t* iters, int32_t* status, float* res, cudaStream_t st);
 int launch_multi(bool adapt, bool exact, bool pull, const MultiArgs& MA, size_t bytes, cudaStream_t st);
+int launch_multi_wide(bool soc, const MultiArgs& MA, int threads, size_t bytes, cudaStream_t st);

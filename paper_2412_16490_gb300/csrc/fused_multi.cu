@@ -26,3 +26,12 @@ int launch_multi(bool adapt, bool exact, bool pull, const MultiArgs& MA, size_t 
   if (exact) return go(multi_kernel<false, true>);
   return adapt ? go(multi_kernel<true>) : go(multi_kernel<false>);
 }
+
+int launch_multi_wide(bool soc, const MultiArgs& MA, int threads, size_t bytes, cudaStream_t st) {
+  auto go = [&](auto kernel) -> int {
+    if (int r = ensure_smem(kernel, bytes)) return r;
+    kernel<<<MA.total, threads, bytes, st>>>(MA);
+    return launch_err("multi_wide_kernel launch");
+  };
+  return soc ? go(multi_wide_kernel<CONE_SOC>) : go(multi_wide_kernel<CONE_PYR>);
+}

@@ -85,3 +85,24 @@ def test_fewer_wrenches_than_contacts(name, tile, solver):
     few = bx.bodex_energy_grad(H, Ob, x, T[:2].contiguous(), sp)
     for k in ("Q", "y"):
         assert torch.equal(few[k], full[k][:, :2]), k
+
+
+@pytest.mark.parametrize("cone", [0, 1])
+@pytest.mark.parametrize("s", [1, 6, 12])
+def test_several_jobs_in_one_wide_launch(cone, s):
+    """Jobs of every contact count in one launch (few QPs: the wide form),
+    bitwise as with a tile asked for (the one-lane form)."""
+    scenes = [_scene(n, B, s, grid=g) for n, B, g in (("hand5", 33, True), ("hand3", 7, False), ("hand4x4", 50, True), ("hand3", 1, True))]
+    outs = []
+    for tile in (0, 8):
+        sp = bx.step_params(I.default_params(), qp=bx.qp_params(max_iter=20, cone=cone), grasps_per_cta=tile)
+        jobs = []
+        for k, (H, Ob, x, T) in enumerate(scenes):
+            st = bx.State(H, x.shape[0], s)
+            st.set_pose(x)
+            jobs.append(dict(hand=H, obj=Ob, state=st, T=T, n_steps=3 + k, E_last=torch.empty(x.shape[0], device="cuda"),
+                             status=torch.empty(x.shape[0], dtype=torch.int32, device="cuda")))
+        bx.bodex_step_multi(jobs, sp)
+        outs.append([t for j in jobs for t in (j["state"].pose(), *j["state"].adam()[:2], j["state"].residual(), j["E_last"], j["status"])])
+    for a, b in zip(*outs):
+        assert torch.equal(a, b)
