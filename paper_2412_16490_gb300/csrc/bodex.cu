@@ -561,7 +561,11 @@ static int upload_spheres(bodex_hand_s* h, const bodex_hand_desc* d) {
   const size_t b_sph = sizeof(float4) * K, b_sb = sizeof(float4) * (n + 1), b_ss = sizeof(int) * (n + 2),
                b_sp = sizeof(int) * (n + 2), b_pa = sizeof(int) * std::max<size_t>(1, spartners.size());
   const size_t o_sb = b_sph, o_ss = o_sb + b_sb, o_sp = o_ss + b_ss, o_pa = o_sp + b_sp;
-  std::vector<char> blob(o_pa + b_pa);
+  const size_t o_sl = o_pa + b_pa;  // each sphere's slot, in slot order
+  std::vector<int> sphere_slot(K);
+  for (int a = 0; a < K; ++a) sphere_slot[a] = slot[order[a]];
+  std::vector<char> blob(o_sl + sizeof(int) * K);
+  std::memcpy(blob.data() + o_sl, sphere_slot.data(), sizeof(int) * K);
   std::memcpy(blob.data(), sph.data(), b_sph);
   std::memcpy(blob.data() + o_sb, sbound.data(), b_sb);
   std::memcpy(blob.data() + o_ss, slot_start.data(), b_ss);
@@ -580,6 +584,7 @@ static int upload_spheres(bodex_hand_s* h, const bodex_hand_desc* d) {
   h->coll.slot_start = reinterpret_cast<const int*>(base + o_ss);
   h->coll.spstart = reinterpret_cast<const int*>(base + o_sp);
   h->coll.spartners = reinterpret_cast<const int*>(base + o_pa);
+  h->coll.sphere_slot = reinterpret_cast<const int*>(base + o_sl);
   return BODEX_OK;
 }
 

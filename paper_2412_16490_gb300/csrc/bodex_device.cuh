@@ -53,6 +53,7 @@ struct CollDev {
   const int* slot_start;
   const int* spstart;
   const int* spartners;
+  const int* sphere_slot;  // [K]
 };
 
 struct CollParams {
@@ -2172,10 +2173,17 @@ __device__ __forceinline__ float penetration_hinge(float p, float eta, float& dh
 // The argument structs are copied into registers first: through references
 // every use would be a local-memory load that stores to shared memory force
 // the compiler to repeat.
-static __device__ __noinline__ void collision_phase(bool active, int lane, int S, const HandDev& H, const CollDev& Cr,
-                                             const ObjDev& Or, const float* x, const CollParams& Pr,
-                                             const float* frames, const float* jw, float* cs, float* sl, float* bw,
-                                             float* gc, float* ep) {
+// With more than S lanes a grasp (LN > S, the wide form) and room for 3 K
+// more words behind bw, the sphere gradients take a lane each (hs: K words):
+// a lane that walked a slot's spheres, up to six of the palm, made a step of
+// 1501 four-finger grasps with 34 spheres 49.8 us; it is 47.0 with a lane a
+// sphere.  The energy is still summed by the first S lanes in the order of
+// their slots, so its bits are the same.
+template <bool WIDE>
+__device__ __forceinline__ void collision_body(bool active, int lane, int S, int LN, int room, const HandDev& H,
+                                               const CollDev& Cr, const ObjDev& Or, const float* x,
+                                               const CollParams& Pr, const float* frames, const float* jw, float* cs,
+                                               float* sl, float* bw, float* hs, float* gc, float* ep) {
   const CollDev C = Cr;
   const ObjDev O = Or;
   const CollParams P = Pr;
@@ -2184,18 +2192,31 @@ static __device__ __noinline__ void collision_phase(bool active, int lane, int S
   // joint-limit term applies.  C.K is uniform, so every thread still meets
   // every barrier below.
   const bool sph = C.K > 0;
+  const bool split = WIDE && 6 * C.K + 9 * nslot <= room;  // uniform
+  const bool first = active && lane < S;  // the lanes that sum the energy
   float e = 0.f;
   // C1: sphere centres from the slot frames
-  if (active && sph)
-    for (int L = lane; L < nslot; L += S) {
-      Tf T;
+  auto slot_frame = [&](int L, Tf& T) {
 #pragma unroll
-      for (int e2 = 0; e2 < 9; ++e2) T.R[e2] = frames[12 * L + e2];
-      T.t[0] = frames[12 * L + 9];
-      T.t[1] = frames[12 * L + 10];
-      T.t[2] = frames[12 * L + 11];
+    for (int e2 = 0; e2 < 9; ++e2) T.R[e2] = frames[12 * L + e2];
+    T.t[0] = frames[12 * L + 9];
+    T.t[1] = frames[12 * L + 10];
+    T.t[2] = frames[12 * L + 11];
+  };
+  if (split && active)
+    for (int k = lane; k < C.K; k += LN) {
+      Tf T;
+      slot_frame(__ldg(C.sphere_slot + k), T);
+      const float4 sp = __ldg(C.sph + k);
+      const float p[3] = {sp.x, sp.y, sp.z};
+      tf_point(T, p, cs + 3 * k);
+    }
+  if (active && sph)
+    for (int L = lane; L < nslot; L += LN) {
+      Tf T;
+      slot_frame(L, T);
       const int k1 = __ldg(C.slot_start + L + 1);
-      for (int k = __ldg(C.slot_start + L); k < k1; ++k) {
+      for (int k = split ? k1 : __ldg(C.slot_start + L); k < k1; ++k) {
         const float4 sp = __ldg(C.sph + k);
         const float p[3] = {sp.x, sp.y, sp.z};
         tf_point(T, p, cs + 3 * k);
@@ -2205,22 +2226,99 @@ static __device__ __noinline__ void collision_phase(bool active, int lane, int S
       tf_point(T, pb, bw + 3 * L);
     }
   __syncthreads();
+  // one overlapping pair of spheres (r1, c) and o: energy and force
+  auto pair = [&](const float* c, float r, int o, float& en, float* f) {
+    const float v[3] = {c[0] - cs[3 * o], c[1] - cs[3 * o + 1], c[2] - cs[3 * o + 2]};
+    const float len2 = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
+    const float rr = r + __ldg(C.sph + o).w;
+    if (len2 < rr * rr) {
+      const float len = sqrtf(len2);
+      const float d = rr - len;
+      en = fmaf(0.5f * P.w_self * d, d, en);  // each pair is visited from both spheres
+      const float sc = -2.f * P.w_self * d / len;
+#pragma unroll
+      for (int a = 0; a < 3; ++a) f[a] = fmaf(sc, v[a], f[a]);
+      return true;
+    }
+    return false;
+  };
+  // whether the bounding spheres of slots L and L2 overlap
+  auto close = [&](int L, int L2) {
+    const float dx = bw[3 * L] - bw[3 * L2], dy = bw[3 * L + 1] - bw[3 * L2 + 1], dz = bw[3 * L + 2] - bw[3 * L2 + 2];
+    const float rr = __ldg(C.sbound + L).w + __ldg(C.sbound + L2).w;
+    return dx * dx + dy * dy + dz * dz < rr * rr;
+  };
+  // the slots whose bounding spheres overlap slot L's, a bit each
+  auto near_slots = [&](int L) {
+    unsigned long long near = 0ull;
+    const int q0 = __ldg(C.spstart + L), q1 = __ldg(C.spstart + L + 1);
+#pragma unroll 4
+    for (int q = q0; q < q1; ++q) {
+      const int L2 = __ldg(C.spartners + q);
+      near |= (unsigned long long)close(L, L2) << L2;
+    }
+    return near;
+  };
+  auto slot_pairs = [&](unsigned long long near, const float* c, float r, float& en, float* f) {
+    bool hit = false;
+    for (; near; near &= near - 1ull) {
+      const int L2 = __ffsll((long long)near) - 1;
+      const int t1 = __ldg(C.slot_start + L2 + 1);
+      for (int o = __ldg(C.slot_start + L2); o < t1; ++o) hit = pair(c, r, o, en, f) || hit;
+    }
+    return hit;
+  };
   // C2: sphere gradients f_k, summed per slot into (F, tau).  Self pairs:
-  // only between slots whose bounding spheres overlap (a mask per slot).
-  if (active && sph)
+  // only between slots whose bounding spheres overlap.
+  float* const fs = bw + 3 * nslot;  // [3 K], split only
+  if (split && active)
+    for (int k = lane; k < C.K; k += LN) {
+      const float c[3] = {cs[3 * k], cs[3 * k + 1], cs[3 * k + 2]};
+      const float r = __ldg(C.sph + k).w;
+      float f[3] = {0.f, 0.f, 0.f}, h = 0.f, en = 0.f;
+      if (P.w_pen != 0.f) {
+        const SdfQ q = sdf_query(O, c);
+        float dh;
+        h = penetration_hinge(r + P.eta_pen - q.phi, P.eta_pen, dh);
+        const float sc = -P.w_pen * dh;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) f[a] = sc * q.g[a];
+      }
+      const bool hit = P.w_self != 0.f && slot_pairs(near_slots(__ldg(C.sphere_slot + k)), c, r, en, f);
+      hs[k] = hit ? -h : h;  // the hinge is never negative: its sign marks a sphere with pairs
+#pragma unroll
+      for (int a = 0; a < 3; ++a) fs[3 * k + a] = f[a];
+    }
+  if (split) __syncthreads();
+  if (split && first && sph)
     for (int L = lane; L < nslot; L += S) {
-      unsigned long long near = 0ull;
-      if (P.w_self != 0.f) {
-        const float4 bL = __ldg(C.sbound + L);
-        const float cL[3] = {bw[3 * L], bw[3 * L + 1], bw[3 * L + 2]};
-        const int q1 = __ldg(C.spstart + L + 1);
-        for (int q = __ldg(C.spstart + L); q < q1; ++q) {
-          const int L2 = __ldg(C.spartners + q);
-          const float dx = cL[0] - bw[3 * L2], dy = cL[1] - bw[3 * L2 + 1], dz = cL[2] - bw[3 * L2 + 2];
-          const float rr = bL.w + __ldg(C.sbound + L2).w;
-          if (dx * dx + dy * dy + dz * dz < rr * rr) near |= 1ull << L2;
+      float F[3] = {0.f, 0.f, 0.f}, tau[3] = {0.f, 0.f, 0.f};
+      const int k1 = __ldg(C.slot_start + L + 1);
+      for (int k = __ldg(C.slot_start + L); k < k1; ++k) {
+        const float c[3] = {cs[3 * k], cs[3 * k + 1], cs[3 * k + 2]}, f[3] = {fs[3 * k], fs[3 * k + 1], fs[3 * k + 2]};
+        const float h = hs[k];
+        if (P.w_pen != 0.f) e = fmaf(P.w_pen, fabsf(h), e);
+        if (signbit(h)) {  // its pairs once more, for the energy in its place
+          float skip[3] = {0.f, 0.f, 0.f};
+          slot_pairs(near_slots(L), c, __ldg(C.sph + k).w, e, skip);
+        }
+        float cf[3];
+        cross3(c, f, cf);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+          F[a] += f[a];
+          tau[a] += cf[a];
         }
       }
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        sl[6 * L + a] = F[a];
+        sl[6 * L + 3 + a] = tau[a];
+      }
+    }
+  if (!split && first && sph)
+    for (int L = lane; L < nslot; L += S) {
+      const unsigned long long near = P.w_self != 0.f ? near_slots(L) : 0ull;
       float F[3] = {0.f, 0.f, 0.f}, tau[3] = {0.f, 0.f, 0.f};
       const int k1 = __ldg(C.slot_start + L + 1);
       for (int k = __ldg(C.slot_start + L); k < k1; ++k) {
@@ -2235,23 +2333,7 @@ static __device__ __noinline__ void collision_phase(bool active, int lane, int S
 #pragma unroll
           for (int a = 0; a < 3; ++a) f[a] = sc * q.g[a];
         }
-        for (unsigned long long m2 = near; m2; m2 &= m2 - 1ull) {
-          const int L2 = __ffsll((long long)m2) - 1;
-          const int t1 = __ldg(C.slot_start + L2 + 1);
-          for (int o = __ldg(C.slot_start + L2); o < t1; ++o) {
-            const float v[3] = {c[0] - cs[3 * o], c[1] - cs[3 * o + 1], c[2] - cs[3 * o + 2]};
-            const float len2 = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
-            const float rr = r + __ldg(C.sph + o).w;
-            if (len2 < rr * rr) {
-              const float len = sqrtf(len2);
-              const float d = rr - len;
-              e = fmaf(0.5f * P.w_self * d, d, e);  // each pair is visited from both spheres
-              const float sc = -2.f * P.w_self * d / len;
-#pragma unroll
-              for (int a = 0; a < 3; ++a) f[a] = fmaf(sc, v[a], f[a]);
-            }
-          }
-        }
+        slot_pairs(near, c, r, e, f);
         float cf[3];
         cross3(c, f, cf);
 #pragma unroll
@@ -2269,17 +2351,23 @@ static __device__ __noinline__ void collision_phase(bool active, int lane, int S
   __syncthreads();
   // C3a: subtree sums, leaves first (parent[j] < j), by one lane; slot n
   // (the root) becomes the total
-  if (active && sph && lane == 0)
-    for (int j = n - 1; j >= 0; --j) {
-      const int p = H.parent[j];
-      const int to = p < 0 ? n : p;
+  // (one component a lane; the one-lane form, with as few lanes as wrenches, all six in lane 0)
+  if (active && sph && lane < (WIDE ? 6 : 1))
+    for (int a0 = lane; a0 < (WIDE ? 6 : 1); a0 += LN)
+      for (int j = n - 1; j >= 0; --j) {
+        const int p = H.parent[j];
+        const int to = p < 0 ? n : p;
+        if (WIDE) {
+          sl[6 * to + a0] += sl[6 * j + a0];
+        } else {
 #pragma unroll
-      for (int a = 0; a < 6; ++a) sl[6 * to + a] += sl[6 * j + a];
-    }
+          for (int a = 0; a < 6; ++a) sl[6 * to + a] += sl[6 * j + a];
+        }
+      }
   __syncthreads();
   // C3b: joint gradients dE/dq_j = w_j . (tau_sub - o_j x F_sub) over the
   // links joint j moves (the root joints: everything), and the limit energy
-  if (active) {
+  if (first) {
     for (int k = lane; k < D; k += S) {
       float g = 0.f;
       if (sph) {
@@ -2330,6 +2418,21 @@ static __device__ __noinline__ void collision_phase(bool active, int lane, int S
     ep[lane] = e;
   }
   __syncthreads();  // the scratch (fr, cs, sl) is reused by the next phase
+}
+
+// The one-lane form's phase and the wide form's, each a call of its own.
+static __device__ __noinline__ void collision_phase(bool active, int lane, int S, const HandDev& H, const CollDev& C,
+                                                    const ObjDev& O, const float* x, const CollParams& P,
+                                                    const float* frames, const float* jw, float* cs, float* sl,
+                                                    float* bw, float* gc, float* ep) {
+  collision_body<false>(active, lane, S, S, 0, H, C, O, x, P, frames, jw, cs, sl, bw, nullptr, gc, ep);
+}
+static __device__ __noinline__ void collision_phase_wide(bool active, int lane, int S, int LN, int room,
+                                                         const HandDev& H, const CollDev& C, const ObjDev& O,
+                                                         const float* x, const CollParams& P, const float* frames,
+                                                         const float* jw, float* cs, float* sl, float* bw, float* hs,
+                                                         float* gc, float* ep) {
+  collision_body<true>(active, lane, S, LN, room, H, C, O, x, P, frames, jw, cs, sl, bw, hs, gc, ep);
 }
 
 }  // namespace bodex

@@ -1270,13 +1270,14 @@ __device__ __forceinline__ void fused_wide_cta(const FusedArgs& A, int cta, int 
       if (st) atomicOr(reinterpret_cast<int*>(per + L::oSC + 1), st);
     }
     __syncthreads();
-    // ---- constraint energies: s lanes, as in fused_cta (the energy is summed lane by lane)
+    // ---- constraint energies on the collision spheres (hinges in the K^-1 block, not yet formed)
+    static_assert(L::KS >= BODEX_MAX_SPHERES, "room for the spheres' hinges");
     if (A.coll) {
       const SetUp u = set_up();
       float* const per = u.per;
-      collision_phase(u.active && u.lane < S, u.lane, S, H, A.cd, A.obj, per + L::oX, A.cp, per + L::oK, per + L::oJW,
-                      per + L::oRY, per + L::oRY + 3 * A.cd.K, per + L::oRY + 3 * A.cd.K + 6 * (H.n + 1),
-                      per + L::oGC, per + L::oGC + MAXD);
+      collision_phase_wide(u.active, u.lane, S, LN, L::COLL_CS, H, A.cd, A.obj, per + L::oX, A.cp, per + L::oK,
+                      per + L::oJW, per + L::oRY, per + L::oRY + 3 * A.cd.K, per + L::oRY + 3 * A.cd.K + 6 * (H.n + 1),
+                      u.kin, per + L::oGC, per + L::oGC + MAXD);
     }
     // ---- A4: K^-1 per grasp
     {
