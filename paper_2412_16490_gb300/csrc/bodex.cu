@@ -1061,7 +1061,7 @@ int bodex_step_multi(const bodex_job* jobs, int n_jobs, const bodex_step_params*
       case 4: threads = std::max(threads, wide_threads<4>(1, J.s)); wide_bytes = std::max(wide_bytes, Lay<4>::bytes(1)); break;
       default: threads = std::max(threads, wide_threads<5>(1, J.s)); wide_bytes = std::max(wide_bytes, Lay<5>::bytes(1)); break;
     }
-    wide_share += (double)S->B * J.s / ((double)wide_limit(m, soc) * sms);
+    wide_share += (double)S->B * J.s / ((double)wide_limit(m, A.cfg, A.coll != 0) * sms);
     tiles[nj] = (S->B + gpb - 1) / gpb;
     // cost of one tile: steps x wrenches x (ADMM work per iteration, 26 m + 9 m^2 + ...,
     // taken as m^2; or m for the exact solve, whose oracle is linear in m)

@@ -1636,25 +1636,33 @@ inline int wide_tile(int s, int B, int sms) {
   return best;
 }
 
-// Whether the fused step runs B grasps of s QPs in the wide form (bitwise the
-// same results).  The wide form's time grows with the QPs per SM; the
-// one-lane form's steps up with each block of 96 lanes that an SM holds.
-// Measured (50 steps of 50 iterations, one-lane -> wide, us), five contacts:
-// 40 QPs an SM 1552 -> 800, 81: 1555 -> 1435, 118: 2334 -> 2089, 162:
-// 2325 -> 2460; four: 118: 1705 -> 1292, 142: 1706 -> 1675, 162:
-// 1700 -> 1871; three: 63: 829 -> 704, 79: 836 -> 875, 103: 1243 -> 877, 162:
-// 1243 -> 1488.  Elliptic cone, whose chain is longer: five contacts 162:
-// 3518 -> 3263, 189: 3521 -> 3497, 237: 4081 -> 4495; four 237: 3027 -> 2595;
-// three 81: 1543 -> 1354, 162: 1826 -> 1859.
-inline int wide_limit(int m, bool soc) {  // in QPs per SM
+// Up to how many QPs per SM the fused step runs in the wide form (bitwise the
+// same results).  The wide form's time grows with the QPs per SM, and its
+// blocks beyond those resident at once (96, 120 and 144 QPs an SM for five,
+// four and three contacts) wait for a second wave; the one-lane form's steps
+// up with each block of 96 lanes that an SM holds.  Measured (50 steps of 50
+// iterations, one-lane -> wide, us), five contacts: 40 QPs an SM 1552 -> 800,
+// 81: 1555 -> 1435, 118: 2334 -> 2089 (of 20 iterations 1268 -> 1351), 162:
+// 2325 -> 2460; four: 81: 1100 -> 1027, 118: 1705 -> 1292, 162: 1700 -> 1871;
+// three: 63: 829 -> 704, 79: 836 -> 875, 103: 1243 -> 877, 162: 1243 -> 1488.
+// Elliptic cone, whose chain is longer: five contacts 162: 3518 -> 3263, 237:
+// 4081 -> 4495; four 237: 3027 -> 2595; three 81: 1543 -> 1354, 162: 1826 ->
+// 1859.  With the collision energies, whose set-up is longer: five 63: 2951 ->
+// 2540, 79: 2903 -> 2966; four 118: 2747 -> 2352, 126: 2662 -> 3372; three 63:
+// 1271 -> 929, 107: 1723 -> 1176; cone, five 96: 4478 -> 3479, 126: 4925 ->
+// 5192; four 118: 3488 -> 2179, 162: 3475 -> 3674; three 118: 2283 -> 1495.
+inline int wide_limit(int m, const AdmmCfg& c, bool coll) {
+  const bool soc = c.cone != 0;
+  if (coll) return soc ? (m == 5 ? 96 : 120) : (m == 5 ? 72 : m == 4 ? 120 : 112);
   if (soc) return m == 5 ? 176 : m == 4 ? 224 : 128;
-  return m == 3 ? 64 : 128;
+  return m == 5 ? (c.iters >= 40 ? 128 : 96) : m == 4 ? 120 : 64;
 }
 template <int M>
-inline bool wide_pays(int s, int B, bool soc, int sms) {
-  const long long n = (long long)B * s;
-  if (M == 3 && !soc && n > 96LL * sms && n <= 112LL * sms) return true;  // a second one-lane block costs more
-  return n <= (long long)wide_limit(M, soc) * sms;
+inline bool wide_pays(const FusedArgs& A, int sms) {
+  const long long n = (long long)A.B * A.S;
+  // three contacts: a second one-lane block an SM costs more
+  if (M == 3 && !A.cfg.cone && n > 96LL * sms && n <= 112LL * sms) return true;
+  return n <= (long long)wide_limit(M, A.cfg, A.coll != 0) * sms;
 }
 
 // Raises the kernel's dynamic shared-memory limit when needed, once per
@@ -1697,7 +1705,7 @@ inline int run_fused(int mode, const FusedArgs& A0, cudaStream_t st) {
   bool wide = mode != MODE_ADJOINT && A.cfg.solver != BODEX_QP_EXACT && !adapt && !A.dfc;
   if (wide) {
     const int sms = sm_count();
-    wide = A.S < M || (A0.gpb <= 0 && wide_pays<M>(A.S, A.B, soc, sms));
+    wide = A.S < M || (A0.gpb <= 0 && wide_pays<M>(A, sms));
     if (wide) A.gpb = wide_tile<M>(A.S, A.B, sms);
   }
   if (!wide) A.gpb = pick_gpb<M>(A.S, A0.gpb);
