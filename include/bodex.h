@@ -247,7 +247,9 @@ typedef struct bodex_step_params {
   float lr_t, lr_r, b1, b2, adam_eps;
   bodex_energy_params energy;
   bodex_qp_params qp;
-  int grasps_per_cta;  /* CTA tile: grasps per thread block (0 = default, 96 / s); an
+  int grasps_per_cta;  /* CTA tile: grasps per thread block (0 = default: 96 / s, or the
+                          form with m lanes per QP where a batch is too small to fill
+                          the GPU; the results are the same); an
                           autotuner knob that changes speed, never results */
   int work_pulling;    /* bodex_step_multi only.  0: one thread block per tile (a job's
                           grasps_per_cta grasps), the jobs' tiles in the caller's order,
