@@ -787,7 +787,7 @@ __device__ __forceinline__ void fused_cta(const FusedArgs& A, int cta, int GPB, 
   // with s < m lanes a grasp, a lane takes several contacts; the
   // fixed-iteration step does without the loop, which cost it 0.8% (13.63
   // against 13.51 ms for 4096 grasps x 200 steps): run_fused gives its s < m
-  // cases to the wide form
+  // cases to the wide form, or under DFC to the kernel with adaptive rho
   constexpr bool ONE_CONTACT = MODE == MODE_STEP && !ADAPT && (CONE == CONE_PYR || CONE == CONE_SOC);
   const HandDev& H = *reinterpret_cast<const HandDev*>(smem);
   float* kin = smem + L::HAND_WORDS + gl * L::KS;
@@ -1700,8 +1700,12 @@ inline int run_fused(int mode, const FusedArgs& A0, cudaStream_t st) {
   FusedArgs A = A0;
   const bool soc = A.cfg.cone != 0;
   const bool adapt = A.cfg.eps > 0.f && A.cfg.adapt;
+  // one lane per QP at a fixed rho takes no fewer wrenches than contacts
+  // (ONE_CONTACT); DFC with fewer runs in the kernel that has the contact
+  // loop, whose lower level it skips
+  const bool any_s = adapt || (A.dfc && A.S < M);
   // the wide form: ADMM at a fixed rho, where it pays and no tile is asked
-  // for, and fewer wrenches than contacts (which the one-lane step does not take)
+  // for, and fewer wrenches than contacts
   bool wide = mode != MODE_ADJOINT && A.cfg.solver != BODEX_QP_EXACT && !adapt && !A.dfc;
   if (wide) {
     const int sms = sm_count();
@@ -1726,8 +1730,8 @@ inline int run_fused(int mode, const FusedArgs& A0, cudaStream_t st) {
   else if (A.cfg.solver == BODEX_QP_EXACT)
     r = mode == MODE_STEP ? go(fused_kernel<M, MODE_STEP, CONE_EXACT, false>) : go(fused_kernel<M, MODE_EVAL, CONE_EXACT, false>);
   else if (mode == MODE_STEP)
-    r = soc ? (adapt ? go(fused_kernel<M, MODE_STEP, CONE_SOC, true>) : go(fused_kernel<M, MODE_STEP, CONE_SOC, false>))
-            : (adapt ? go(fused_kernel<M, MODE_STEP, CONE_PYR, true>) : go(fused_kernel<M, MODE_STEP, CONE_PYR, false>));
+    r = soc ? (any_s ? go(fused_kernel<M, MODE_STEP, CONE_SOC, true>) : go(fused_kernel<M, MODE_STEP, CONE_SOC, false>))
+            : (any_s ? go(fused_kernel<M, MODE_STEP, CONE_PYR, true>) : go(fused_kernel<M, MODE_STEP, CONE_PYR, false>));
   else
     r = soc ? (adapt ? go(fused_kernel<M, MODE_EVAL, CONE_SOC, true>) : go(fused_kernel<M, MODE_EVAL, CONE_SOC, false>))
             : (adapt ? go(fused_kernel<M, MODE_EVAL, CONE_PYR, true>) : go(fused_kernel<M, MODE_EVAL, CONE_PYR, false>));

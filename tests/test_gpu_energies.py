@@ -94,3 +94,34 @@ def test_qp_baseline_beta_zero_matches_oracle():
     g, gref = host(out["dEdx"]), ev["grad"]
     rel = np.linalg.norm(g - gref, axis=1) / np.maximum(np.linalg.norm(gref, axis=1), 1e-3)
     assert (rel[ok] <= 1e-3).all(), rel[ok].max()
+
+
+@pytest.mark.parametrize("kind,s", [("tiny", 1), ("tiny", 2), ("tiny", 3), ("paper", 1), ("paper", 2), ("paper", 4), ("paper", 5)])
+@pytest.mark.parametrize("collide", [False, True])
+def test_dfc_step_with_fewer_wrenches_than_contacts(kind, s, collide):
+    """The DFC energy does not depend on the wrenches, and a step places every
+    contact however few of them there are: one step is Adam on the gradient,
+    E the oracle's.  A CTA holds several grasps (s lanes each), the last one
+    fewer."""
+    B = 53
+    hand, obj, x0, T, P = _workload(kind, B)
+    coll = dict(w_pen=2.0, w_self=5.0, w_lim=1.0, eta_pen=0.005, eta_lim=0.2) if collide else {}
+    H, Ob = bx.Hand(hand), bx.Object(obj)
+    sp = bx.step_params(dict(P, energy=bx.ENERGY_DFC, **coll))
+    x = cuda(x0)
+    few = cuda(T[:s])
+    g = host(bx.bodex_energy_grad(H, Ob, x, few, sp)["dEdx"])
+    st = bx.State(H, B, s)
+    st.set_pose(x)
+    E = torch.empty(B, device="cuda")
+    # other grasps' contacts at the same place of shared memory, so that a contact the step leaves out shows
+    bx.bodex_energy_grad(H, Ob, x.roll(1, 0).contiguous(), few, sp)
+    bx.bodex_step(H, Ob, st, few, 1, sp, E_last=E)
+    lr = np.where(np.arange(hand.dof) < 3, P["lr_t"], P["lr_r"])
+    want = np.clip(x0 - lr * g / (np.abs(g) + P["adam_eps"]), hand.qmin, hand.qmax)
+    # Adam's first step is lr * sign(g): a tiny gradient may differ in sign between the two kernels
+    big = np.abs(g) > 1e-3 * np.abs(g).max(1, keepdims=True)
+    np.testing.assert_allclose(host(st.pose())[big], want[big], atol=2e-6)
+    ev = O.evaluate(O.Hand(hand), O.Object(obj), x0.astype(np.float64), T[:s], dict(P, energy=O.ENERGY_DFC, **coll))
+    ok = _off_faces(obj, ev["c"]).all(-1) if obj.kind != "sphere" else np.ones(B, bool)
+    np.testing.assert_allclose(host(E)[ok], ev["E"][ok], rtol=1e-4, atol=1e-6)
