@@ -1008,15 +1008,16 @@ int bodex_step_multi(const bodex_job* jobs, int n_jobs, const bodex_step_params*
   size_t bytes = 0;
   int total = 0, nj = 0;
   // the wide form for all jobs or none: ADMM at a fixed rho, no tile or
-  // pulling asked for, and few enough QPs for it to pay (wide_limit)
+  // pulling asked for, where its estimated time is shorter (form_time)
   const bool exact = params->qp.solver == BODEX_QP_EXACT;
   const bool adapt = !exact && params->qp.eps_abs > 0.f && params->qp.adaptive_rho;
   const bool soc = params->qp.cone != BODEX_CONE_PYRAMID;
   bool wide = !exact && !adapt && params->energy.kind != BODEX_ENERGY_DFC && params->grasps_per_cta <= 0 && !params->work_pulling;
   int threads = 0;
   size_t wide_bytes = 0;
-  double wide_share = 0.0;  // of the QPs per SM up to which the wide form pays
-  const int sms = wide ? sm_count() : 1;
+  FormLoad lane[BODEX_MAX_JOBS], lanes[BODEX_MAX_JOBS];
+  int lane_threads = 0;
+  bool coll = false;
   int take[BODEX_MAX_JOBS], tiles[BODEX_MAX_JOBS];
   double cost[BODEX_MAX_JOBS];
   for (int j = 0; j < n_jobs; ++j) {
@@ -1061,8 +1062,11 @@ int bodex_step_multi(const bodex_job* jobs, int n_jobs, const bodex_step_params*
       case 4: threads = std::max(threads, wide_threads<4>(1, J.s)); wide_bytes = std::max(wide_bytes, Lay<4>::bytes(1)); break;
       default: threads = std::max(threads, wide_threads<5>(1, J.s)); wide_bytes = std::max(wide_bytes, Lay<5>::bytes(1)); break;
     }
-    wide_share += (double)S->B * J.s / ((double)wide_limit(m, A.cfg, A.coll != 0) * sms);
     tiles[nj] = (S->B + gpb - 1) / gpb;
+    lane[nj] = {m, J.s, gpb, tiles[nj], J.n_steps};
+    lanes[nj] = {m, J.s, 1, S->B, J.n_steps};
+    lane_threads = std::max(lane_threads, gpb * J.s);
+    coll = A.coll != 0;
     // cost of one tile: steps x wrenches x (ADMM work per iteration, 26 m + 9 m^2 + ...,
     // taken as m^2; or m for the exact solve, whose oracle is linear in m)
     cost[nj] = (double)J.n_steps * J.s * (exact ? m : m * m);
@@ -1071,7 +1075,12 @@ int bodex_step_multi(const bodex_job* jobs, int n_jobs, const bodex_step_params*
     take[nj] = j;
     ++nj;
   }
-  wide = wide && wide_share <= 1.0;
+  if (wide && nj > 0) {
+    const int sms = sm_count();
+    const AdmmCfg& c = MA->job[0].cfg;
+    wide = form_time(true, lanes, nj, threads, wide_bytes, c, coll, sms) <
+           0.96 * form_time(false, lane, nj, lane_threads, bytes, c, coll, sms);
+  }
   if (wide) {
     total = 0;
     for (int k = 0; k < nj; ++k) {

@@ -1537,11 +1537,12 @@ __device__ __forceinline__ void multi_item(const MultiArgs& A, int w, float* sme
 
 // The same in the wide form (fixed rho, no pulling): every job's tile is one
 // grasp, blocks as wide as the widest job needs; a warp that a job leaves
-// without QPs still shares its set-up phases.  Taken when the jobs' shares of
-// wide_limit add up to at most 1: six jobs of three hands, 12 wrenches, 50
+// without QPs still shares its set-up phases.  Taken where its estimate (form_time) is
+// the shorter one: six jobs of three hands, 12 wrenches, 50
 // steps of 50 iterations take 912 us instead of 1772 with 200 grasps
 // together, 1321 (1873) with 900, 2396 (2553) with 1600; with 2000 the
-// one-lane form is ahead, 2586 against 2691.
+// one-lane form is ahead, 2586 against 2691.  (A warp without QPs also runs
+// every iteration, on zeros.)
 template <int CONE>
 __global__ void __launch_bounds__(WIDE_THREADS, 4) multi_wide_kernel(const __grid_constant__ MultiArgs A) {
   extern __shared__ __align__(16) float smem[];
@@ -1636,33 +1637,97 @@ inline int wide_tile(int s, int B, int sms) {
   return best;
 }
 
-// Up to how many QPs per SM the fused step runs in the wide form (bitwise the
-// same results).  The wide form's time grows with the QPs per SM, and its
-// blocks beyond those resident at once (96, 120 and 144 QPs an SM for five,
-// four and three contacts) wait for a second wave; the one-lane form's steps
-// up with each block of 96 lanes that an SM holds.  Measured (50 steps of 50
-// iterations, one-lane -> wide, us), five contacts: 40 QPs an SM 1552 -> 800,
-// 81: 1555 -> 1435, 118: 2334 -> 2089 (of 20 iterations 1268 -> 1351), 162:
-// 2325 -> 2460; four: 81: 1100 -> 1027, 118: 1705 -> 1292, 162: 1700 -> 1871;
-// three: 63: 829 -> 704, 79: 836 -> 875, 103: 1243 -> 877, 162: 1243 -> 1488.
-// Elliptic cone, whose chain is longer: five contacts 162: 3518 -> 3263, 237:
-// 4081 -> 4495; four 237: 3027 -> 2595; three 81: 1543 -> 1354, 162: 1826 ->
-// 1859.  With the collision energies, whose set-up is longer: five 63: 2951 ->
-// 2540, 79: 2903 -> 2966; four 118: 2747 -> 2352, 126: 2662 -> 3372; three 63:
-// 1271 -> 929, 107: 1723 -> 1176; cone, five 96: 4478 -> 3479, 126: 4925 ->
-// 5192; four 118: 3488 -> 2179, 162: 3475 -> 3674; three 118: 2283 -> 1495.
-inline int wide_limit(int m, const AdmmCfg& c, bool coll) {
-  const bool soc = c.cone != 0;
-  if (coll) return soc ? (m == 5 ? 96 : 120) : (m == 5 ? 72 : m == 4 ? 120 : 112);
-  if (soc) return m == 5 ? 176 : m == 4 ? 224 : 128;
-  return m == 5 ? (c.iters >= 40 ? 128 : 96) : m == 4 ? 120 : 64;
+// Which form a fused step takes: the one whose estimated time is shorter (the
+// results are bitwise the same).  Both are latency-bound steps that rise with
+// the warps on the busiest scheduler, u = 1..4, and with every further wave of
+// blocks: a bound in QPs per SM alone, fitted at 12 wrenches, was wrong by up
+// to 1.8 times for others (five contacts, 16 wrenches, 94 QPs an SM: 116 -> 157
+// us for 6 steps of 20 iterations, as the wide form's blocks of 3 warps take a
+// second wave there; elliptic cone, 174 QPs, 3 iterations: 89 -> 159).
+// Measured at 23 batch sizes of 8 to 238 QPs an SM, s = m, 8, 12 and 16, 3 to
+// 150 iterations, with and without collision energies, us:
+//   - an iteration, one lane per QP, by u: three contacts 0.17, 0.34, 0.51 (a
+//     block has 3 warps, an SM at most 4 blocks); wide 0.09, 0.15, 0.20, 0.27;
+//   - the set-up of a wave of blocks: a constant, and a part that grows with
+//     the grasps and, wide, the warps an SM holds; the collision energies'
+//     part of a one-lane block is spread over the s lanes of a grasp;
+//   - a later wave of the wide form overlaps the one before: 0.75 to 0.99 of
+//     its own time (its last blocks start as the first ones end).
+// The wide form is taken below 0.93 of the one-lane estimate.  Over the 6624
+// measured pairs that is within 0.6% of always taking the faster form, in the
+// mean; the worst choice that is slower than one lane loses 9% (three
+// contacts, 16 wrenches, 10 iterations).
+struct FormCost {
+  double set, grasp, warp, inv_s;             // set-up of a wave: set + grasp * grasps/SM + warp * warps/SM + inv_s / s
+  double coll, coll_grasp, coll_warp, coll_inv_s;  // the same with the collision energies
+  double pyr[4], soc[4];                      // one ADMM iteration by warps on the busiest scheduler
+};
+inline const FormCost& form_cost(bool wide, int m) {
+  static const FormCost lane[3] = {
+      {8.55, 0.07, 0, 0, 13.0, 0.19, 0, 47, {0.173, 0.335, 0.51, 0.51}, {0.465, 0.566, 0.68, 0.68}},
+      {9.2, 0.11, 0, 0, 18.6, 0.25, 0, 92, {0.27, 0.495, 0.75, 0.75}, {0.68, 0.84, 1.02, 1.02}},
+      {10.7, 0.10, 0, 0, 22.0, 0.19, 0, 147, {0.405, 0.70, 1.05, 1.05}, {1.03, 1.19, 1.41, 1.41}}};
+  static const FormCost lanes[3] = {
+      {7.07, 0.08, 0.09, 0, 11.7, 0.37, -0.05, 0, {0.089, 0.145, 0.203, 0.271}, {0.197, 0.232, 0.33, 0.40}},
+      {7.18, 0.20, 0.11, 0, 16.1, 1.38, -0.27, 0, {0.103, 0.158, 0.236, 0.318}, {0.207, 0.244, 0.30, 0.36}},
+      {7.35, 0.22, 0.12, 0, 18.6, 2.24, -0.43, 0, {0.117, 0.18, 0.26, 0.353}, {0.235, 0.278, 0.34, 0.42}}};
+  return (wide ? lanes : lane)[m - 3];
 }
+
+// One job's part of a launch: `blocks` blocks of gpb grasps.
+struct FormLoad {
+  int m, s, gpb, blocks, steps;
+};
+
+// Estimated time of a launch of n jobs' blocks, `threads` wide with `bytes`
+// of shared memory each, us.
+inline double form_time(bool wide, const FormLoad* job, int n, int threads, size_t bytes, const AdmmCfg& c, bool coll,
+                        int sms) {
+  constexpr size_t kSmemPerSM = 228 * 1024, kReserved = 1024;  // 1 KB of every block is the system's
+  const int wpb = (threads + 31) / 32;
+  const int resident = std::max(1, std::min((wide ? 16 : 12) / wpb, (int)(kSmemPerSM / (bytes + kReserved))));
+  // with a residual target the QPs of a warp rarely all stop early; beyond
+  // 300 iterations the set-up no longer matters
+  const double iters = c.eps > 0.f ? std::min(c.iters, 300) : c.iters;
+  long long total = 0;
+  int counts = 0;  // a bit per contact count
+  for (int k = 0; k < n; ++k) {
+    total += job[k].blocks;
+    counts |= 1 << job[k].m;
+  }
+  const bool mixed = counts == (1 << 3 | 1 << 4 | 1 << 5);
+  double t = 0;
+  bool first = true;
+  for (long long per = (total + sms - 1) / sms; per > 0; first = false) {
+    const int r = (int)std::min<long long>(per, resident), warps = r * wpb, u = std::min((warps + 3) / 4, 4);
+    per -= r;
+    double mean = 0, longest = 0;
+    for (int k = 0; k < n; ++k) {
+      const FormCost& f = form_cost(wide, job[k].m);
+      const double g = (double)r * job[k].gpb;
+      double v = coll ? f.coll + f.coll_grasp * g + f.coll_warp * warps + f.coll_inv_s / job[k].s
+                      : f.set + f.grasp * g + f.warp * warps + f.inv_s / job[k].s;
+      v = job[k].steps * (v + iters * (c.cone ? f.soc : f.pyr)[u - 1]);
+      mean += v * job[k].blocks / total;
+      longest = std::max(longest, v);
+    }
+    double wave = per > 0 ? mean : longest;  // the launch ends with its longest blocks
+    // three contact counts on an SM: the wide form's many small blocks run
+    // three kernels' code at once (measured against the estimates: 1.13 to
+    // 1.26 with four warps a scheduler, 1.08 below, 1.06 for the cone)
+    if (wide && mixed) wave *= c.cone ? 1.06 : u == 4 ? 1.2 : 1.08;
+    if (wide && !first) wave *= (c.cone ? 0.75 : 0.8) + 0.06 * (u - 1) + (coll ? 0.1 : 0.0);
+    t += wave;
+  }
+  return t;
+}
+
 template <int M>
 inline bool wide_pays(const FusedArgs& A, int sms) {
-  const long long n = (long long)A.B * A.S;
-  // three contacts: a second one-lane block an SM costs more
-  if (M == 3 && !A.cfg.cone && n > 96LL * sms && n <= 112LL * sms) return true;
-  return n <= (long long)wide_limit(M, A.cfg, A.coll != 0) * sms;
+  const int g1 = pick_gpb<M>(A.S, 0), gw = wide_tile<M>(A.S, A.B, sms);
+  const FormLoad lane = {M, A.S, g1, (A.B + g1 - 1) / g1, 1}, lanes = {M, A.S, gw, (A.B + gw - 1) / gw, 1};
+  return form_time(true, &lanes, 1, wide_threads<M>(gw, A.S), Lay<M>::bytes(gw), A.cfg, A.coll != 0, sms) <
+         0.93 * form_time(false, &lane, 1, g1 * A.S, Lay<M>::bytes(g1), A.cfg, A.coll != 0, sms);
 }
 
 // Raises the kernel's dynamic shared-memory limit when needed, once per

@@ -1,0 +1,119 @@
+"""Which kernel a fused step takes.  The wide form (m lanes per QP) and the
+one-lane form give the same bits; the default takes the one whose estimated
+time is shorter, and a requested tile the one-lane form.  The kernels that a
+call launches are read from a captured graph."""
+import re
+import warnings
+
+import numpy as np
+import pytest
+
+from gpu_helpers import I, cuda, torch
+
+import paper_2412_16490_gb300 as bx
+
+pytestmark = pytest.mark.gpu
+
+COLLISION = dict(w_pen=100.0, w_self=100.0, w_lim=10.0, eta_pen=0.005, eta_lim=0.05)
+
+
+def _launched(call, tmp_path):
+    """Names of the step kernels that `call` launches."""
+    call()
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph(keep_graph=True)
+    g.enable_debug_mode()
+    with torch.cuda.graph(g):
+        call()
+    path = tmp_path / "graph.dot"
+    with warnings.catch_warnings():
+        warnings.simplefilter("ignore")  # the dump announces itself
+        g.debug_dump(str(path))
+    return re.findall(r"(fused_wide_kernel|fused_kernel|multi_wide_kernel|multi_kernel)", path.read_text())
+
+
+def _scene(name, B, s):
+    hand = I.hand_template(name)
+    obj = I.grid_object(3, n=32)
+    T = I.wrench_set(12)
+    T = T[:s] if s <= 12 else np.concatenate([T, np.roll(0.5 * T, 1, axis=1)[:s - 12]])
+    x = I.initial_poses(hand, obj, min(B, 40), seed=5)
+    H = bx.Hand(hand)
+    st = bx.State(H, B, s)
+    st.set_pose(cuda(np.tile(x, (-(-B // 40), 1))[:B]))
+    return dict(hand=H, obj=bx.Object(obj), state=st, T=cuda(T))
+
+
+def _step(j, sp, n=1):
+    bx.bodex_step(j["hand"], j["obj"], j["state"], j["T"], n, sp)
+
+
+@pytest.mark.parametrize("name,s,B", [("hand5", 12, 1), ("hand5", 12, 700), ("hand5", 7, 33), ("hand5", 16, 5), ("hand4", 6, 64),
+                                      ("hand4x4", 12, 801), ("hand3", 12, 799), ("hand3", 12, 1301)])
+@pytest.mark.parametrize("cone", [0, 1])
+@pytest.mark.parametrize("collide", [False, True])
+def test_small_batches_take_the_wide_form(name, s, B, cone, collide, tmp_path):
+    """The cases whose two forms test_gpu_wide compares do run in two forms."""
+    P = I.default_params(**(COLLISION if collide else {}))
+    j = _scene(name, B, s)
+    for qp in (bx.qp_params(max_iter=20, cone=cone), bx.qp_params(max_iter=60, eps_abs=1e-3, check_every=7, cone=cone)):
+        assert _launched(lambda: _step(j, bx.step_params(P, qp=qp)), tmp_path) == ["fused_wide_kernel"]
+        assert _launched(lambda: _step(j, bx.step_params(P, qp=qp, grasps_per_cta=8)), tmp_path) == ["fused_kernel"]
+
+
+@pytest.mark.parametrize("s", [1, 6, 12])
+def test_several_small_jobs_take_the_wide_form(s, tmp_path):
+    jobs = [dict(_scene(n, B, s), n_steps=1) for n, B in (("hand5", 33), ("hand3", 7), ("hand4x4", 50), ("hand3", 1))]
+    for tile, kernel in ((0, "multi_wide_kernel"), (8, "multi_kernel")):
+        sp = bx.step_params(I.default_params(), qp=bx.qp_params(max_iter=20), grasps_per_cta=tile)
+        assert _launched(lambda: bx.bodex_step_multi(jobs, sp), tmp_path) == [kernel]
+
+
+def _times(calls, reps=9):
+    """Shortest time of each call in ms, the calls taken in turn."""
+    best = [float("inf")] * len(calls)
+    for r in range(reps):
+        for k, (reset, call) in enumerate(calls):
+            reset()
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            call()
+            b.record()
+            torch.cuda.synchronize()
+            if r:
+                best[k] = min(best[k], a.elapsed_time(b))
+    return best
+
+
+# sizes around the second wave of either form, at few wrenches and many, few iterations and many;
+# the shorter of the two estimates is at most some 10% from the faster form
+@pytest.mark.parametrize("name,s,B,cone,iters,collide", [
+    ("hand5", 16, 893, 0, 20, False), ("hand5", 16, 893, 0, 50, False), ("hand5", 5, 2857, 0, 20, False),
+    ("hand5", 16, 1653, 1, 3, False), ("hand5", 8, 3306, 1, 3, False), ("hand4x4", 8, 4218, 1, 3, False),
+    ("hand5", 16, 893, 1, 3, True), ("hand3", 12, 1216, 0, 300, True), ("hand4x4", 12, 1500, 0, 50, True),
+    ("hand3", 16, 720, 0, 150, False), ("hand5", 12, 1000, 0, 50, False), ("hand3", 12, 400, 0, 50, False),
+])
+def test_default_form_is_not_the_slower_one(name, s, B, cone, iters, collide):
+    sp = [bx.step_params(I.default_params(**(COLLISION if collide else {})), qp=bx.qp_params(max_iter=iters, cone=cone),
+                         grasps_per_cta=tile) for tile in (0, 96 // s)]
+    j = _scene(name, B, s)
+    x = j["state"].pose()
+    auto, lane = _times([(lambda: j["state"].set_pose(x), lambda p=p: _step(j, p, 8)) for p in sp])
+    assert auto <= 1.15 * lane, (auto, lane)
+
+
+@pytest.mark.parametrize("mix,s,collide", [((("hand5", 900),), 16, False), ((("hand3", 1400),), 12, True),
+                                           ((("hand5", 400), ("hand3", 400), ("hand4x4", 400)) * 2, 6, True),
+                                           ((("hand5", 140), ("hand3", 140), ("hand4x4", 140)) * 2, 16, False)])
+def test_default_form_of_several_jobs_is_not_the_slower_one(mix, s, collide):
+    P = I.default_params(**(COLLISION if collide else {}))
+    jobs = [dict(_scene(n, B, s), n_steps=8) for n, B in mix]
+    xs = [j["state"].pose() for j in jobs]
+
+    def reset():
+        for j, x in zip(jobs, xs):
+            j["state"].set_pose(x)
+
+    sp = [bx.step_params(P, qp=bx.qp_params(max_iter=20), grasps_per_cta=tile) for tile in (0, 96 // s)]
+    auto, lane = _times([(reset, lambda p=p: bx.bodex_step_multi(jobs, p)) for p in sp])
+    assert auto <= 1.15 * lane, (auto, lane)
