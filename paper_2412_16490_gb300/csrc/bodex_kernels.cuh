@@ -775,7 +775,7 @@ __device__ __forceinline__ void assemble_step(const FusedArgs& A, const HandDev&
   }
 }
 
-template <int M, int MODE, int CONE = CONE_ANY, bool ADAPT = false>
+template <int M, int MODE, int CONE = CONE_ANY, bool ADAPT = false, bool FEW = false>
 __device__ __forceinline__ void fused_cta(const FusedArgs& A, int cta, int GPB, float* smem) {
   using L = Lay<M>;
   constexpr int NV = L::NV, NC = L::NC;
@@ -784,11 +784,15 @@ __device__ __forceinline__ void fused_cta(const FusedArgs& A, int cta, int GPB, 
   const int gl = threadIdx.x / S, lane = threadIdx.x % S;
   const int b = cta * GPB + gl;
   const bool active = (gl < GPB) && (b < A.B);
-  // with s < m lanes a grasp, a lane takes several contacts; the
-  // fixed-iteration step does without the loop, which cost it 0.8% (13.63
-  // against 13.51 ms for 4096 grasps x 200 steps): run_fused gives its s < m
-  // cases to the wide form, or under DFC to the kernel with adaptive rho
-  constexpr bool ONE_CONTACT = MODE == MODE_STEP && !ADAPT && (CONE == CONE_PYR || CONE == CONE_SOC);
+  // With s < m lanes a grasp, a lane takes several contacts.  The kernels of
+  // one cone do without that loop, which cost the fixed-iteration step 0.8%
+  // (13.63 against 13.51 ms for 4096 grasps x 200 steps), the adaptive one of
+  // five contacts 5% (310 -> 326 us for 3 steps of 2000 grasps) and its
+  // evaluation 10% (349 -> 385 us at 810 grasps), where it spills the iterate
+  // (816 bytes of loads instead of 384): run_fused gives their s < m cases to
+  // the wide form or, with adaptive rho and under DFC, to the kernels for few
+  // wrenches (FEW).
+  constexpr bool ONE_CONTACT = !FEW && MODE != MODE_ADJOINT && (CONE == CONE_PYR || CONE == CONE_SOC);
   const HandDev& H = *reinterpret_cast<const HandDev*>(smem);
   float* kin = smem + L::HAND_WORDS + gl * L::KS;
   float* per = smem + L::HAND_WORDS + GPB * L::KS + gl * L::PER;
@@ -1132,10 +1136,10 @@ __device__ __forceinline__ void fused_cta(const FusedArgs& A, int cta, int GPB, 
   }
 }
 
-template <int M, int MODE, int CONE, bool ADAPT>
+template <int M, int MODE, int CONE, bool ADAPT, bool FEW = false>
 __global__ void __launch_bounds__(CTA_LANES, 4) fused_kernel(FusedArgs A) {
   extern __shared__ __align__(16) float smem[];
-  fused_cta<M, MODE, CONE, ADAPT>(A, blockIdx.x, A.gpb, smem);
+  fused_cta<M, MODE, CONE, ADAPT, FEW>(A, blockIdx.x, A.gpb, smem);
 }
 
 // ============================================================================ kernel: fused evaluation / step, wide form
@@ -1765,16 +1769,13 @@ inline int run_fused(int mode, const FusedArgs& A0, cudaStream_t st) {
   FusedArgs A = A0;
   const bool soc = A.cfg.cone != 0;
   const bool adapt = A.cfg.eps > 0.f && A.cfg.adapt;
-  // one lane per QP at a fixed rho takes no fewer wrenches than contacts
-  // (ONE_CONTACT); DFC with fewer runs in the kernel that has the contact
-  // loop, whose lower level it skips
-  const bool any_s = adapt || (A.dfc && A.S < M);
+  const bool few = A.S < M;  // fewer wrenches than contacts: not in the one-lane kernels of one cone (ONE_CONTACT)
   // the wide form: ADMM at a fixed rho, where it pays and no tile is asked
   // for, and fewer wrenches than contacts
   bool wide = mode != MODE_ADJOINT && A.cfg.solver != BODEX_QP_EXACT && !adapt && !A.dfc;
   if (wide) {
     const int sms = sm_count();
-    wide = A.S < M || (A0.gpb <= 0 && wide_pays<M>(A, sms));
+    wide = few || (A0.gpb <= 0 && wide_pays<M>(A, sms));
     if (wide) A.gpb = wide_tile<M>(A.S, A.B, sms);
   }
   if (!wide) A.gpb = pick_gpb<M>(A.S, A0.gpb);
@@ -1794,9 +1795,12 @@ inline int run_fused(int mode, const FusedArgs& A0, cudaStream_t st) {
     r = soc ? go(fused_wide_kernel<M, MODE_EVAL, CONE_SOC>) : go(fused_wide_kernel<M, MODE_EVAL, CONE_PYR>);
   else if (A.cfg.solver == BODEX_QP_EXACT)
     r = mode == MODE_STEP ? go(fused_kernel<M, MODE_STEP, CONE_EXACT, false>) : go(fused_kernel<M, MODE_EVAL, CONE_EXACT, false>);
+  else if (few)  // adaptive rho, or DFC, which skips the lower level
+    r = soc ? (mode == MODE_STEP ? go(fused_kernel<M, MODE_STEP, CONE_SOC, true, true>) : go(fused_kernel<M, MODE_EVAL, CONE_SOC, true, true>))
+            : (mode == MODE_STEP ? go(fused_kernel<M, MODE_STEP, CONE_PYR, true, true>) : go(fused_kernel<M, MODE_EVAL, CONE_PYR, true, true>));
   else if (mode == MODE_STEP)
-    r = soc ? (any_s ? go(fused_kernel<M, MODE_STEP, CONE_SOC, true>) : go(fused_kernel<M, MODE_STEP, CONE_SOC, false>))
-            : (any_s ? go(fused_kernel<M, MODE_STEP, CONE_PYR, true>) : go(fused_kernel<M, MODE_STEP, CONE_PYR, false>));
+    r = soc ? (adapt ? go(fused_kernel<M, MODE_STEP, CONE_SOC, true>) : go(fused_kernel<M, MODE_STEP, CONE_SOC, false>))
+            : (adapt ? go(fused_kernel<M, MODE_STEP, CONE_PYR, true>) : go(fused_kernel<M, MODE_STEP, CONE_PYR, false>));
   else
     r = soc ? (adapt ? go(fused_kernel<M, MODE_EVAL, CONE_SOC, true>) : go(fused_kernel<M, MODE_EVAL, CONE_SOC, false>))
             : (adapt ? go(fused_kernel<M, MODE_EVAL, CONE_PYR, true>) : go(fused_kernel<M, MODE_EVAL, CONE_PYR, false>));
