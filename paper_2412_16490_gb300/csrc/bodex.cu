@@ -154,16 +154,21 @@ __global__ void __launch_bounds__(FkTile<M>::THREADS) fk_contacts_kernel(const H
 //   E = w_d sum |c^{f'} - (p^f + delta n_out)|^2 + w_qp sum |c^{f'} - p^c|^2
 // with p^f, n_out and the coarse-stage points p^c treated as constants.
 // delta is the pre-grasp margin (Sec. IV-D): 1 cm in the fine stage, 0 in
-// the final one.  One warp per grasp and RF_GPB warps a block, with no block
-// barrier between steps: lanes 0..m-1 own a contact's kinematics and adjoint,
-// all 32 lanes share each fingertip's samples (the queries are most of the
-// work: 160 a grasp and step), the gradient assembly and Adam; the chains are
-// walked by three lanes a contact, one row of the frames each, and the lowest
-// sample found by two warp reductions (4096 grasps x 100 steps: 1.50 -> 1.37
-// ms together).  With eight
-// lanes a grasp and each contact's samples walked by one of them, a step of
-// 4096 grasps was bound by the latency of 32 queries in a row on 6.7 warps an
-// SM.
+// the final one.  Lanes 0..m-1 own a contact's adjoint, all lanes of a grasp
+// share the gradient assembly and Adam, and no block barrier stands between
+// steps.  Two forms:
+//   - a warp per grasp: all 32 lanes share each fingertip's samples (160
+//     queries a grasp and step with 32 samples), the chains are walked by
+//     three lanes a contact, one row of the frames each, and the lowest sample
+//     is found by two warp reductions.  A step of 4096 five-finger grasps in a
+//     64^3 grid takes 14.3 us, with eight lanes 34.6: those are bound by the
+//     latency of 32 queries in a row;
+//   - eight lanes per grasp: a lane walks its contact's chain and samples.  A
+//     warp holds four grasps' serial parts, so where the queries are few or
+//     cheap and the batch fills the GPU it is the shorter one: 16,384 grasps
+//     with 7 samples 24 us a step instead of 42, on a sphere object with 32
+//     samples 14.0 instead of 23.2.
+// warp_per_grasp chooses.  Both find the same sample and give the same bits.
 struct RefineArgs {
   const HandDev* hand;
   const float* tips;
@@ -173,6 +178,7 @@ struct RefineArgs {
   float delta, w_d, w_qp;
   float lr_t, lr_r, b1, b2, adam_eps;
   int n_steps, t0;
+  int S;  // samples per fingertip
   float* x;
   float* am;
   float* av;
@@ -181,7 +187,8 @@ struct RefineArgs {
   int32_t* status;
 };
 
-constexpr int RF_GPB = 4;  // grasps (warps) per block of the refinement and metrics kernels
+// The refinement and metrics kernels: blocks of 128 threads, LANES (32 or 8) a grasp.
+constexpr int RF_THREADS = 128;
 
 // The fingertip sample with the smallest phi over the warp, lowest index on
 // ties (0 if none compares below infinity): T is the contact's link frame.
@@ -221,16 +228,38 @@ __device__ __forceinline__ void load_frame(const float* f, Tf& T) {
   T.t[2] = f[11];
 }
 
-template <int M>
-__global__ void __launch_bounds__(32 * RF_GPB) refine_kernel(RefineArgs A) {
-  constexpr int HW = Lay<M>::HAND_WORDS;
+// Contact i's samples walked by one lane: the smallest phi (infinity if none
+// compares below it) and the lowest index that has it.
+__device__ __forceinline__ int lowest_sample_lane(const Tf& T, const float* __restrict__ tip, int S, const ObjDev& obj,
+                                                  float& phi) {
+  phi = INFINITY;
+  int kbest = 0;
+  for (int k = 0; k < S; ++k) {
+    const float sk[3] = {__ldg(tip + 3 * k), __ldg(tip + 3 * k + 1), __ldg(tip + 3 * k + 2)};
+    float ck[3];
+    tf_point(T, sk, ck);
+    const float ph = sdf_query(obj, ck).phi;
+    if (ph < phi) {
+      phi = ph;
+      kbest = k;
+    }
+  }
+  return kbest;
+}
+
+template <int M, int LANES>
+__global__ void __launch_bounds__(RF_THREADS) refine_kernel(RefineArgs A) {
+  constexpr bool WARP = LANES == 32;  // else a lane walks its contact's chain and samples
+  constexpr int HW = Lay<M>::HAND_WORDS, GPB = RF_THREADS / LANES;
   constexpr int CBW = 6 + MAXCHAIN;
-  constexpr int oRQ = 3 * MAXD + M * CBW + M * MAXCHAIN * 6 + M * 12 + M + 1;  // joint rotations and the root frame
-  constexpr int PER = align4(oRQ + 9 * MAXJ + 12 + 4);
-  __shared__ __align__(16) float smem[HW + RF_GPB * PER];
+  constexpr int oEi = 3 * MAXD + M * CBW + M * MAXCHAIN * 6 + (WARP ? M * 12 : 0);
+  constexpr int oRQ = oEi + M + 1;  // joint rotations and the root frame (WARP)
+  constexpr int PER = align4(oRQ + (WARP ? 9 * MAXJ + 12 : 0) + 4);
+  __shared__ __align__(16) float smem[HW + GPB * PER];
   copy_hand_to_smem(A.hand, smem);
-  const int gl = threadIdx.x / 32, lane = threadIdx.x % 32;
-  const int b = blockIdx.x * RF_GPB + gl;
+  const int gl = threadIdx.x / LANES, lane = threadIdx.x % LANES;
+  const int b_mine = blockIdx.x * GPB + gl;
+  const int b = min(b_mine, A.B - 1);  // a group past the last grasp repeats it and writes nothing
   const HandDev& H = *reinterpret_cast<const HandDev*>(smem);
   float* per = smem + HW + gl * PER;
   float* xs = per;
@@ -238,13 +267,13 @@ __global__ void __launch_bounds__(32 * RF_GPB) refine_kernel(RefineArgs A) {
   float* avs = per + 2 * MAXD;
   float* cb = per + 3 * MAXD;
   float* jwall = cb + M * CBW;
-  float* frames = jwall + M * MAXCHAIN * 6;
-  float* Ei = frames + M * 12;
+  float* frames = jwall + M * MAXCHAIN * 6;  // WARP
+  float* Ei = per + oEi;
   int* stat = reinterpret_cast<int*>(Ei + M);
   __syncthreads();
-  if (b >= A.B) return;  // whole warps; no block barrier below
+  if (b_mine - (int)(threadIdx.x % 32) / LANES >= A.B) return;  // whole warps; no block barrier below
   const int D = H.D, S = H.S;
-  for (int k = lane; k < D; k += 32) {
+  for (int k = lane; k < D; k += LANES) {
     xs[k] = A.x[(size_t)b * D + k];
     ams[k] = A.am[(size_t)b * D + k];
     avs[k] = A.av[(size_t)b * D + k];
@@ -253,24 +282,29 @@ __global__ void __launch_bounds__(32 * RF_GPB) refine_kernel(RefineArgs A) {
   __syncwarp();
   int kbest = 0;
   for (int step = 0; step < A.n_steps; ++step) {
-    const float* jw = jwall + (lane < M ? lane : 0) * MAXCHAIN * 6;
-    for (int e = lane; e <= H.n; e += 32) fk_joint(H, e, xs, per + oRQ, per + oRQ + 9 * MAXJ);
-    __syncwarp();
-    if (lane < 3 * M)
-      fk_row(H, lane / 3, lane % 3, per + oRQ, per + oRQ + 9 * MAXJ, jwall + (lane / 3) * MAXCHAIN * 6, nullptr,
-             frames + 12 * (lane / 3), nullptr);
-    __syncwarp();
+    float* const jw = jwall + (lane < M ? lane : 0) * MAXCHAIN * 6;
+    Tf T;  // lane < M: contact lane's link frame
+    if constexpr (WARP) {
+      for (int e = lane; e <= H.n; e += 32) fk_joint(H, e, xs, per + oRQ, per + oRQ + 9 * MAXJ);
+      __syncwarp();
+      if (lane < 3 * M)
+        fk_row(H, lane / 3, lane % 3, per + oRQ, per + oRQ + 9 * MAXJ, jwall + (lane / 3) * MAXCHAIN * 6, nullptr,
+               frames + 12 * (lane / 3), nullptr);
+      __syncwarp();
 #pragma unroll
-    for (int i = 0; i < M; ++i) {
-      Tf T;
-      load_frame(frames + 12 * i, T);
+      for (int i = 0; i < M; ++i) {
+        load_frame(frames + 12 * i, T);
+        float phi;
+        const int k = lowest_sample(T, A.tips + (size_t)i * S * 3, S, A.obj, phi);
+        if (lane == i) kbest = k;
+      }
+      if (lane < M) load_frame(frames + 12 * lane, T);
+    } else if (lane < M) {
+      fk_link(H, lane, xs, T, jw);
       float phi;
-      const int k = lowest_sample(T, A.tips + (size_t)i * S * 3, S, A.obj, phi);
-      if (lane == i) kbest = k;
+      kbest = lowest_sample_lane(T, A.tips + (size_t)lane * S * 3, S, A.obj, phi);
     }
     if (lane < M) {
-      Tf T;
-      load_frame(frames + 12 * lane, T);
       const float* tip = A.tips + (size_t)lane * S * 3;
       const float sk[3] = {__ldg(tip + 3 * kbest), __ldg(tip + 3 * kbest + 1), __ldg(tip + 3 * kbest + 2)};
       float cf[3];
@@ -299,7 +333,7 @@ __global__ void __launch_bounds__(32 * RF_GPB) refine_kernel(RefineArgs A) {
         for (int i = 0; i < M; ++i) e += Ei[i];
         per[PER - 1] = e;
       }
-      for (int k = lane; k < D; k += 32) {
+      for (int k = lane; k < D; k += LANES) {
         float g = 0.f;
         if (k < 6) {
 #pragma unroll
@@ -326,7 +360,8 @@ __global__ void __launch_bounds__(32 * RF_GPB) refine_kernel(RefineArgs A) {
     }
     __syncwarp();
   }
-  for (int k = lane; k < D; k += 32) {
+  if (b_mine >= A.B) return;
+  for (int k = lane; k < D; k += LANES) {
     A.x[(size_t)b * D + k] = xs[k];
     A.am[(size_t)b * D + k] = ams[k];
     A.av[(size_t)b * D + k] = avs[k];
@@ -341,67 +376,77 @@ __global__ void __launch_bounds__(32 * RF_GPB) refine_kernel(RefineArgs A) {
 // ============================================================================ kernel: contact metrics
 // Contact Distance Consistency (Sec. V-B): d_i = the signed distance of
 // fingertip i, the smallest phi over its surface samples (phi(c_i) - alpha
-// for a hand without samples); cdc = max_i d_i - min_i d_i.  One warp per
-// grasp: lanes 0..m-1 place their links, then the warp shares each finger's
-// samples (with one lane a finger, walking its 32 samples: 59 us for 16,384
-// five-finger poses).
+// for a hand without samples); cdc = max_i d_i - min_i d_i.  In the two forms
+// of the refinement: with a warp per grasp 4096 five-finger poses with 32
+// samples take 20 us (eight lanes 37), 16,384 poses 48 (60); with eight lanes
+// 16,384 poses with 7 samples 22 (35).
 struct MetricsArgs {
   const HandDev* hand;
   const float* tips;  // [m, S, 3] or null
   ObjDev obj;
   int B;
+  int S;  // samples per fingertip, 0 without
   const float* x;
   float* d;    // [B, m]
   float* cdc;  // [B], may be null
 };
 
-template <int M>
-__global__ void __launch_bounds__(32 * RF_GPB) metrics_kernel(MetricsArgs A) {
-  constexpr int HW = Lay<M>::HAND_WORDS;
-  constexpr int oRQ = align4(MAXD) + 12 * M;  // joint rotations and the root frame
-  constexpr int PER = oRQ + 9 * MAXJ + 12;
-  __shared__ __align__(16) float smem[HW + RF_GPB * PER];
+template <int M, int LANES>
+__global__ void __launch_bounds__(RF_THREADS) metrics_kernel(MetricsArgs A) {
+  constexpr bool WARP = LANES == 32;
+  constexpr int HW = Lay<M>::HAND_WORDS, GPB = RF_THREADS / LANES;
+  constexpr int oRQ = align4(MAXD) + 12 * M;  // joint rotations and the root frame (WARP)
+  constexpr int PER = WARP ? oRQ + 9 * MAXJ + 12 : align4(MAXD);
+  __shared__ __align__(16) float smem[HW + GPB * PER];
   copy_hand_to_smem(A.hand, smem);
-  const int gl = threadIdx.x / 32, lane = threadIdx.x % 32;
-  const int b = blockIdx.x * RF_GPB + gl;
+  const int gl = threadIdx.x / LANES, lane = threadIdx.x % LANES;
+  const int b_mine = blockIdx.x * GPB + gl;
+  const int b = min(b_mine, A.B - 1);  // a group past the last grasp repeats it and writes nothing
   const HandDev& H = *reinterpret_cast<const HandDev*>(smem);
   float* xs = smem + HW + gl * PER;
-  float* frames = xs + align4(MAXD);
+  float* frames = xs + align4(MAXD);  // WARP
   __syncthreads();
-  if (b >= A.B) return;  // whole warps; no block barrier below
+  if (b_mine - (int)(threadIdx.x % 32) / LANES >= A.B) return;  // whole warps; no block barrier below
   const int D = H.D, S = A.tips ? H.S : 0;
-  for (int k = lane; k < D; k += 32) xs[k] = A.x[(size_t)b * D + k];
-  __syncwarp();
-  for (int e = lane; e <= H.n; e += 32) fk_joint(H, e, xs, xs + oRQ, xs + oRQ + 9 * MAXJ);
-  __syncwarp();
-  if (lane < 3 * M)
-    fk_row(H, lane / 3, lane % 3, xs + oRQ, xs + oRQ + 9 * MAXJ, nullptr, nullptr, frames + 12 * (lane / 3), nullptr);
+  for (int k = lane; k < D; k += LANES) xs[k] = A.x[(size_t)b * D + k];
   __syncwarp();
   float d = 0.f;
-  if (S > 0) {
+  Tf T;  // lane < M: contact lane's link frame
+  if constexpr (WARP) {
+    for (int e = lane; e <= H.n; e += 32) fk_joint(H, e, xs, xs + oRQ, xs + oRQ + 9 * MAXJ);
+    __syncwarp();
+    if (lane < 3 * M)
+      fk_row(H, lane / 3, lane % 3, xs + oRQ, xs + oRQ + 9 * MAXJ, nullptr, nullptr, frames + 12 * (lane / 3), nullptr);
+    __syncwarp();
+    if (S > 0) {
 #pragma unroll
-    for (int i = 0; i < M; ++i) {
-      Tf T;
-      load_frame(frames + 12 * i, T);
-      float phi;
-      (void)lowest_sample(T, A.tips + (size_t)i * S * 3, S, A.obj, phi);
-      if (lane == i) d = phi;
+      for (int i = 0; i < M; ++i) {
+        load_frame(frames + 12 * i, T);
+        float phi;
+        (void)lowest_sample(T, A.tips + (size_t)i * S * 3, S, A.obj, phi);
+        if (lane == i) d = phi;
+      }
+    } else if (lane < M) {
+      load_frame(frames + 12 * lane, T);
     }
   } else if (lane < M) {
-    Tf T;
-    load_frame(frames + 12 * lane, T);
+    fk_link(H, lane, xs, T, nullptr);
+    if (S > 0) (void)lowest_sample_lane(T, A.tips + (size_t)lane * S * 3, S, A.obj, d);
+  }
+  if (S == 0 && lane < M) {
     float c[3];
     tf_point(T, H.clocal[lane], c);
     d = sdf_query(A.obj, c).phi - H.alpha;
   }
-  if (lane < M) A.d[(size_t)b * M + lane] = d;
-  // spread over the grasp's fingers (in the lowest eight lanes)
+  // spread over the grasp's fingers (in its lowest eight lanes)
   float lo = lane < M ? d : INFINITY, hi = lane < M ? d : -INFINITY;
 #pragma unroll
   for (int off = 4; off >= 1; off >>= 1) {
     lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, off));
     hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, off));
   }
+  if (b_mine >= A.B) return;
+  if (lane < M) A.d[(size_t)b * M + lane] = d;
   if (lane == 0 && A.cdc) A.cdc[b] = hi - lo;
 }
 
@@ -446,17 +491,40 @@ int run_fk(const bodex_hand_s* h, const bodex_object_s* o, const float* x, int B
 }  // namespace
 
 namespace {
+// Whether refinement and metrics take a warp per grasp: above a number of
+// samples a finger that grows with the grasps an SM holds (g) until the batch
+// fills the GPU.  Measured at 64 to 65,536 grasps and 1 to 128 samples, us a
+// step, eight lanes -> a warp.  64^3 grid, five fingers: 2000 grasps, 2
+// samples 5.9 -> 7.6, 4: 7.6 -> 7.7, 8: 11.1 -> 7.9; 6000 grasps, 8: 14.6 ->
+// 18.9, 12: 19.2 -> 19.3, 16: 24.1 -> 19.9; 65,536 grasps, 12: 136 -> 165,
+// 16: 194 -> 170 (three fingers 16: 83 -> 107, 24: 115 -> 113; the metrics
+// cross at some 20 for every hand, hence `most`).  Sphere, whose queries are
+// arithmetic alone: 2000 grasps, 12: 4.3 -> 4.4, 24: 5.3 -> 4.3; 6000, 32: 8.0
+// -> 9.9, 48: 9.5 -> 11.4, 64: 11.6 -> 11.3; 65,536, 64: 76 -> 102, 128: 128
+// -> 127.  More than 32 samples are two and more rounds of the warp.
+template <int M>
+bool warp_per_grasp(const ObjDev& obj, int S, int B, double most) {
+  const double g = (double)B / sm_count(), rounds = S > 32 ? 0.8 * S : S;
+  return rounds > (obj.kind == 0 ? std::min(std::max(1.0, g), 80.0) : std::min(std::max(2.0, 0.27 * g), most));
+}
+
 template <int M>
 int run_refine(const RefineArgs& A, cudaStream_t st) {
   (void)cudaGetLastError();
-  refine_kernel<M><<<(A.B + RF_GPB - 1) / RF_GPB, 32 * RF_GPB, 0, st>>>(A);
+  if (warp_per_grasp<M>(A.obj, A.S, A.B, 64.0 / M))
+    refine_kernel<M, 32><<<(A.B + RF_THREADS / 32 - 1) / (RF_THREADS / 32), RF_THREADS, 0, st>>>(A);
+  else
+    refine_kernel<M, 8><<<(A.B + RF_THREADS / 8 - 1) / (RF_THREADS / 8), RF_THREADS, 0, st>>>(A);
   return launch_err("refine_kernel launch");
 }
 
 template <int M>
 int run_metrics(const MetricsArgs& A, cudaStream_t st) {
   (void)cudaGetLastError();
-  metrics_kernel<M><<<(A.B + RF_GPB - 1) / RF_GPB, 32 * RF_GPB, 0, st>>>(A);
+  if (warp_per_grasp<M>(A.obj, A.S, A.B, 20.0))
+    metrics_kernel<M, 32><<<(A.B + RF_THREADS / 32 - 1) / (RF_THREADS / 32), RF_THREADS, 0, st>>>(A);
+  else
+    metrics_kernel<M, 8><<<(A.B + RF_THREADS / 8 - 1) / (RF_THREADS / 8), RF_THREADS, 0, st>>>(A);
   return launch_err("metrics_kernel launch");
 }
 }  // namespace
@@ -1151,6 +1219,7 @@ extern "C" int bodex_refine(bodex_hand_t h, bodex_object_t o, bodex_state_t S, c
   A.adam_eps = p->adam_eps;
   A.n_steps = n_steps;
   A.t0 = S->t;
+  A.S = h->host.S;
   A.x = S->x;
   A.am = S->am;
   A.av = S->av;
@@ -1180,6 +1249,7 @@ extern "C" int bodex_contact_metrics(bodex_hand_t h, bodex_object_t o, const flo
   A.tips = (h->host.S > 0) ? h->tips : nullptr;
   A.obj = o->dev;
   A.B = B;
+  A.S = A.tips ? h->host.S : 0;
   A.x = x;
   A.d = d;
   A.cdc = cdc;
