@@ -379,7 +379,14 @@ __global__ void __launch_bounds__(CTA_LANES, 4) qp_solve_kernel(const float* __r
         park_store(threadIdx.x);
       }
       rebuild();
-      if (mine) park_load(threadIdx.x);
+      if (mine) {
+        park_load(threadIdx.x);
+      } else {  // nothing of an idle thread lives across the rebuild
+#pragma unroll
+        for (int a = 0; a < NV; ++a) y[a] = mq[a] = 0.f;
+#pragma unroll
+        for (int k = 0; k < NC; ++k) w[k] = 0.f;
+      }
     }
   }
   compact();
@@ -421,7 +428,10 @@ __global__ void __launch_bounds__(CTA_LANES, 4) qp_solve_kernel(const float* __r
       const float* Gg = per(g) + L::oG;
       // running QPs advance in lockstep rounds, so they share `it`
       const int chunk = __reduce_max_sync(0xffffffffu, mine ? min(check, cfg.iters - it) : 0);
-#pragma unroll 1
+      // two at a time with adaptive rho: one by one, five contacts' shuffles were
+      // scheduled each before its own multiply-adds (0.29 us an iteration, two
+      // at a time 0.14, the fixed-rho kernel 0.11)
+#pragma unroll (ADAPT ? 2 : 1)
       for (int k = 0; k < chunk; ++k) W.iterate(cfg, rho, gb);
       it += chunk;
       float rpg, rdg, scale[2] = {0.f, 0.f};  // scales: adaptive rho only
@@ -469,7 +479,7 @@ __global__ void __launch_bounds__(CTA_LANES, 4) qp_solve_kernel(const float* __r
         W.wsum = rescale_sum_row(W.wsum, ratio, cfg.gamma);
       }
       rebuild();
-      if (p >= 0) W.load_rows(kin(p / S), ci);  // every group: the rows need not live across the rebuild
+      W.load_rows(kin(max(p, 0) / S), ci);  // every lane: the rows need not live across the rebuild
     }
     if ((n_run + L::QPW - 1) / L::QPW < ww) {
       // fewer warps hold the rest: their state through the parking area, in
