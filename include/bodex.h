@@ -439,11 +439,13 @@ int bodex_squeeze_pose(const float* x, const float* x_p, int B, int D, float* x_
  *     (cudaGetSymbolAddress) with that device current; make that first call
  *     before any stream capture.  Under CUDA's default lazy module loading
  *     that first call (and the first call with a hand of a new contact
- *     count m, whose kernel lives in another module) also loads the
+ *     count m, whose kernels live in another module) also loads the
  *     library's code and the array onto the device, which does allocate
  *     device memory: a caller with a no-allocation phase makes one warm-up
  *     call per device and per hand template at start-up, before that phase.
- *     Calls after the warm-up allocate nothing.
+ *     It loads every kernel that a step of that hand can run, so calls after
+ *     the warm-up allocate nothing, whatever their batch, wrenches and
+ *     parameters.
  *   - All calls share the array and each clears what it uses before its
  *     kernel runs: calls that overlap on the GPU (other streams, other host
  *     threads) race and must be serialised by the caller.

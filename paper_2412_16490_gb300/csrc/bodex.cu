@@ -1296,14 +1296,19 @@ constexpr size_t kNoallocScratchFloats = size_t(1) << 20;  // 4 MiB per device
 constexpr int kNoallocMaxDevices = 64;
 std::mutex g_noalloc_mu;
 float* g_noalloc_addr[kNoallocMaxDevices] = {};
+bool g_noalloc_loaded[kNoallocMaxDevices][MAXM + 1] = {};  // the step kernels of m contacts
 }  // namespace
 
 static __device__ __align__(256) float g_noalloc_scratch[kNoallocScratchFloats];
 
 // Device address of the scratch array on the current device.  Host code may
 // not use the symbol itself (it names a host-side stand-in), so the address
-// is looked up once per device, with that device current, and cached.
-static int noalloc_scratch(float** out) {
+// is looked up once per device, with that device current, and cached.  The
+// first call with a contact count also loads every step kernel of that count:
+// which one runs depends on the batch, the wrenches and the parameters, and
+// lazy loading would take device memory at the first launch of each (2 MB at
+// the first large batch after a warm-up with a small one).
+static int noalloc_scratch(int m, float** out) {
   int dev = 0;
   BODEX_CUDA(cudaGetDevice(&dev));
   if (dev < 0 || dev >= kNoallocMaxDevices) return fail(BODEX_ERR_INVALID, "device ordinal out of range");
@@ -1313,6 +1318,10 @@ static int noalloc_scratch(float** out) {
     cudaError_t e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
     if (e != cudaSuccess) return cuda_fail(e, "cudaGetSymbolAddress(g_noalloc_scratch)");
     g_noalloc_addr[dev] = static_cast<float*>(p);
+  }
+  if (!g_noalloc_loaded[dev][m]) {
+    if (int r = m == 3 ? load_steps_m3() : m == 4 ? load_steps_m4() : load_steps_m5()) return r;
+    g_noalloc_loaded[dev][m] = true;
   }
   *out = g_noalloc_addr[dev];
   return BODEX_OK;
@@ -1335,7 +1344,7 @@ extern "C" int bodex_step_noalloc(bodex_hand_t h, bodex_object_t o, float* x, in
                 "(1048576 floats); use bodex_state_create + bodex_step for larger batches");
   if (n_steps == 0 || B == 0) return BODEX_OK;
   float* base = nullptr;
-  if (int r = noalloc_scratch(&base)) return r;
+  if (int r = noalloc_scratch((int)m, &base)) return r;
   cudaStream_t st = as_stream(stream);
   // the array keeps the previous call's contents: Adam moments and warm
   // starts must start at zero

@@ -1773,6 +1773,18 @@ inline int ensure_smem(K kernel, size_t bytes) {
 
 }  // namespace bodex
 
+// The kernel of a step or an evaluation.
+using FusedKernel = void (*)(FusedArgs);
+template <int M, int MODE>
+inline FusedKernel fused_for(bool wide, bool exact, bool few, bool adapt, bool soc) {
+  if (wide) return soc ? fused_wide_kernel<M, MODE, CONE_SOC> : fused_wide_kernel<M, MODE, CONE_PYR>;
+  if (exact) return fused_kernel<M, MODE, CONE_EXACT, false>;
+  if (few)  // adaptive rho, or DFC, which skips the lower level
+    return soc ? fused_kernel<M, MODE, CONE_SOC, true, true> : fused_kernel<M, MODE, CONE_PYR, true, true>;
+  if (adapt) return soc ? fused_kernel<M, MODE, CONE_SOC, true> : fused_kernel<M, MODE, CONE_PYR, true>;
+  return soc ? fused_kernel<M, MODE, CONE_SOC, false> : fused_kernel<M, MODE, CONE_PYR, false>;
+}
+
 template <int M>
 inline int run_fused(int mode, const FusedArgs& A0, cudaStream_t st) {
   if (A0.B == 0) return BODEX_OK;
@@ -1792,30 +1804,25 @@ inline int run_fused(int mode, const FusedArgs& A0, cudaStream_t st) {
   const int gpb = A.gpb;
   const size_t bytes = Lay<M>::bytes(gpb);
   const dim3 grid((A.B + gpb - 1) / gpb), block(wide ? wide_threads<M>(gpb, A.S) : gpb * A.S);
-  auto go = [&](auto kernel) -> int {
-    if (int r = ensure_smem(kernel, bytes)) return r;
-    kernel<<<grid, block, bytes, st>>>(A);
-    return BODEX_OK;
-  };
-  int r;
-  if (mode == MODE_ADJOINT) r = go(fused_kernel<M, MODE_ADJOINT, CONE_PYR, false>);  // no lower-level solve
-  else if (wide && mode == MODE_STEP)
-    r = soc ? go(fused_wide_kernel<M, MODE_STEP, CONE_SOC>) : go(fused_wide_kernel<M, MODE_STEP, CONE_PYR>);
-  else if (wide)
-    r = soc ? go(fused_wide_kernel<M, MODE_EVAL, CONE_SOC>) : go(fused_wide_kernel<M, MODE_EVAL, CONE_PYR>);
-  else if (A.cfg.solver == BODEX_QP_EXACT)
-    r = mode == MODE_STEP ? go(fused_kernel<M, MODE_STEP, CONE_EXACT, false>) : go(fused_kernel<M, MODE_EVAL, CONE_EXACT, false>);
-  else if (few)  // adaptive rho, or DFC, which skips the lower level
-    r = soc ? (mode == MODE_STEP ? go(fused_kernel<M, MODE_STEP, CONE_SOC, true, true>) : go(fused_kernel<M, MODE_EVAL, CONE_SOC, true, true>))
-            : (mode == MODE_STEP ? go(fused_kernel<M, MODE_STEP, CONE_PYR, true, true>) : go(fused_kernel<M, MODE_EVAL, CONE_PYR, true, true>));
-  else if (mode == MODE_STEP)
-    r = soc ? (adapt ? go(fused_kernel<M, MODE_STEP, CONE_SOC, true>) : go(fused_kernel<M, MODE_STEP, CONE_SOC, false>))
-            : (adapt ? go(fused_kernel<M, MODE_STEP, CONE_PYR, true>) : go(fused_kernel<M, MODE_STEP, CONE_PYR, false>));
-  else
-    r = soc ? (adapt ? go(fused_kernel<M, MODE_EVAL, CONE_SOC, true>) : go(fused_kernel<M, MODE_EVAL, CONE_SOC, false>))
-            : (adapt ? go(fused_kernel<M, MODE_EVAL, CONE_PYR, true>) : go(fused_kernel<M, MODE_EVAL, CONE_PYR, false>));
-  if (r) return r;
+  const bool exact = A.cfg.solver == BODEX_QP_EXACT;
+  const FusedKernel kernel = mode == MODE_ADJOINT ? fused_kernel<M, MODE_ADJOINT, CONE_PYR, false>  // no lower-level solve
+                             : mode == MODE_STEP  ? fused_for<M, MODE_STEP>(wide, exact, few, adapt, soc)
+                                                  : fused_for<M, MODE_EVAL>(wide, exact, few, adapt, soc);
+  if (int r = ensure_smem(kernel, bytes)) return r;
+  kernel<<<grid, block, bytes, st>>>(A);
   return launch_err("fused_kernel launch");
+}
+
+// Puts the code of every step kernel of M contacts on the current device.
+template <int M>
+inline int load_steps() {
+  for (int k = 0; k < 32; ++k) {
+    cudaFuncAttributes a;
+    const cudaError_t e =
+        cudaFuncGetAttributes(&a, fused_for<M, MODE_STEP>(k & 1, (k & 2) != 0, (k & 4) != 0, (k & 8) != 0, (k & 16) != 0));
+    if (e != cudaSuccess) return cuda_fail(e, "cudaFuncGetAttributes(step kernel)");
+  }
+  return BODEX_OK;
 }
 
 template <int M>
@@ -1867,6 +1874,9 @@ inline int run_qp(const float* G, int B, const float* T, int s, const AdmmCfg& c
 int launch_fused_m3(int mode, const FusedArgs& A, cudaStream_t st);
 int launch_fused_m4(int mode, const FusedArgs& A, cudaStream_t st);
 int launch_fused_m5(int mode, const FusedArgs& A, cudaStream_t st);
+int load_steps_m3();
+int load_steps_m4();
+int load_steps_m5();
 int launch_qp(int m, const float* G, int B, const float* T, int s, const AdmmCfg& cfg, int warm, float* y, float* z,
               float* lam, float* Q, int32_t* iters, int32_t* status, float* res, cudaStream_t st);
 int launch_multi(bool adapt, bool exact, bool pull, const MultiArgs& MA, size_t bytes, cudaStream_t st);

@@ -80,3 +80,52 @@ def test_noalloc_step_refuses_batches_beyond_its_array():
                                 None, C.c_void_p(torch.cuda.current_stream().cuda_stream))
     assert rc == _binding.BODEX_ERR_INVALID
     assert b"scratch" in lib.bodex_last_error()
+
+
+LAZY = """
+import ctypes as C, sys
+import numpy as np, torch
+import bodex_inputs as I
+import paper_2412_16490_gb300 as bx
+lib = bx.load()
+ptr = lambda t: C.c_void_p(t.data_ptr())
+hand, obj = I.hand_template(sys.argv[1]), I.grid_object(3, n=32)
+H, Ob = bx.Hand(hand), bx.Object(obj)
+x = torch.as_tensor(np.tile(I.initial_poses(hand, obj, 40, seed=5), (40, 1)).astype(np.float32)).cuda()
+T = torch.as_tensor(I.wrench_set(12).astype(np.float32)).cuda()
+E, status = torch.empty(1600, device="cuda"), torch.empty(1600, dtype=torch.int32, device="cuda")
+P = I.default_params()
+coll = dict(P, w_pen=100.0, w_self=100.0, w_lim=10.0, eta_pen=0.005, eta_lim=0.05)
+
+def taken(B, s, P, tile=0, **qp):
+    sp = bx.step_params(P, qp=bx.qp_params(max_iter=20, **qp), grasps_per_cta=tile)
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    rc = lib.bodex_step_noalloc(H.handle, Ob.handle, ptr(x), B, ptr(T), s, 2, C.byref(sp), ptr(E), ptr(status),
+                                C.c_void_p(torch.cuda.current_stream().cuda_stream))
+    assert rc == 0, lib.bodex_last_error()
+    torch.cuda.synchronize()
+    return free - torch.cuda.mem_get_info()[0]
+
+taken(4, 12, P)  # the warm-up
+calls = [(4, 12, P, {}), (1300, 12, P, {}), (4, 12, P, dict(tile=4)), (4, 2, P, {}), (4, 12, P, dict(cone=1)), (1300, 12, P, dict(cone=1, tile=4)),
+         (4, 12, P, dict(solver=bx.QP_EXACT)), (4, 12, coll, {}), (700, 12, coll, dict(tile=4))]
+for cone in (0, 1):
+    for s in (2, 12):
+        calls += [(30, s, P, dict(cone=cone, eps_abs=1e-4, adaptive_rho=1)), (30, s, dict(P, energy=bx.ENERGY_DFC), dict(cone=cone))]
+got = [taken(B, s, Q, **kw) for B, s, Q, kw in calls]
+assert not any(got), list(zip(got, calls))
+"""
+
+
+@pytest.mark.parametrize("name", ["hand3", "hand4x4", "hand5"])
+def test_one_small_warm_up_covers_every_step(name):
+    """A fresh process under lazy loading: after one small warm-up call no
+    batch size, wrench count, solver, cone or energy takes device memory."""
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    env = dict(os.environ, CUDA_MODULE_LOADING="LAZY", PYTHONPATH=root)
+    run = subprocess.run([sys.executable, "-c", LAZY, name], cwd=root, env=env, capture_output=True, text=True, timeout=300)
+    assert run.returncode == 0, run.stderr[-2000:]
