@@ -4,7 +4,10 @@ Two knobs change how fast the step runs:
 
 * the CTA tile, grasps per thread block (s lanes each): smaller tiles give
   more CTAs, so the grid spreads more evenly over the 152 SMs, at the price
-  of partly filled warps (the tile never changes results);
+  of partly filled warps (the tile never changes results).  Tile 0 leaves the
+  choice to the library, which for ADMM at a fixed rho and a batch too small
+  to fill the GPU takes the form with m lanes per QP; a requested tile runs
+  one lane per QP;
 * the lower-level schedule per upper step: ADMM with a fixed iteration
   count; ADMM to the 1e-5 residual up to a cap, warm-started from the
   previous upper step, its residuals checked every 10 or 25 iterations
@@ -21,7 +24,9 @@ returns the fastest acceptable one.  Two rules of acceptance:
   solve's Frank-Wolfe gap, an upper bound on Q - Q*).
 
 Every candidate's time, median energy and residual fraction are reported.
-Results are cached per (template, wrench count, batch bucket, rule).
+Results are cached per (template, wrench count, batch bucket, rule); a key
+also names the candidate set, so that a file written when there were fewer
+candidates is tuned again.
 """
 from __future__ import annotations
 
@@ -33,7 +38,7 @@ import numpy as np
 
 from . import QP_EXACT, State, bodex_step, qp_params, step_params
 
-TILES = (2, 4, 8)
+TILES = (0, 2, 4, 8)
 SCHEDULES = (
     dict(mode="fixed", iters=20),
     dict(mode="fixed", iters=30),
@@ -44,6 +49,8 @@ SCHEDULES = (
     dict(mode="exact", cap=64),
 )
 REFERENCE = dict(mode="fixed", iters=50)
+
+CANDIDATES = "t0"  # in every key: changed with TILES and SCHEDULES
 
 _cache: dict = {}
 _lock = threading.Lock()
@@ -63,7 +70,7 @@ def schedule_qp(sched: dict, base: dict | None = None):
 
 def key_for(hand, s: int, B: int, residual=None) -> str:
     rule = "energy" if residual is None else f"res{residual:g}"
-    return f"m{hand.m}-n{hand.n}-s{s}-B{1 << max(0, int(np.ceil(np.log2(max(B, 1)))))}-{rule}"
+    return f"m{hand.m}-n{hand.n}-s{s}-B{1 << max(0, int(np.ceil(np.log2(max(B, 1)))))}-{rule}-{CANDIDATES}"
 
 
 def autotune(hand, obj, x0, T, params: dict, steps: int = 200, energy_tol: float = 0.01, reps: int = 2,

@@ -51,3 +51,34 @@ def test_autotune_picks_fastest_accepted_and_reproduces_it(residual):
     # a second call with the same key returns the cached choice without timing again
     assert AT.autotune(H, Ob, x0, T, P, steps=steps, reps=1, tiles=TILES, schedules=SCHEDULES,
                        residual=residual) is out
+
+
+def test_small_batch_is_tuned_no_slower_than_the_default(tmp_path):
+    """A batch that leaves the GPU idle runs fastest without a requested tile
+    (m lanes per QP): the tuner tries that too, and a cache file from before it
+    did is not taken."""
+    import json
+    AT._cache.clear()
+    H, Ob, x0, T, P = _workload()
+    sched = dict(mode="fixed", iters=30)
+    cache = tmp_path / "tuned.json"
+    old = f"m{H.m}-n{H.n}-s{T.shape[0]}-B64-energy"
+    cache.write_text(json.dumps({old: dict(key=old, grasps_per_cta=8, schedule=sched, ms=0.0)}))
+    out = AT.autotune(H, Ob, x0, T, P, steps=50, reps=3, schedules=(sched,), reference=sched, cache_path=str(cache))
+    assert {t["tile"] for t in out["table"]} == set(AT.TILES)
+    ms = []
+    for sp in (AT.tuned_params(out, P), bx.step_params(P, qp=AT.schedule_qp(sched, P))):
+        best = float("inf")
+        for r in range(8):
+            st = bx.State(H, x0.shape[0], T.shape[0])
+            st.set_pose(x0)
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            bx.bodex_step(H, Ob, st, T, 50, sp)
+            b.record()
+            torch.cuda.synchronize()
+            if r:
+                best = min(best, a.elapsed_time(b))
+        ms.append(best)
+    assert ms[0] <= 1.25 * ms[1], ms
+    assert set(json.loads(cache.read_text())) == {old, out["key"]}
