@@ -2,13 +2,14 @@
 one-lane form give the same bits; the default takes the one whose estimated
 time is shorter, and a requested tile the one-lane form.  The kernels that a
 call launches are read from a captured graph."""
+import dataclasses
 import re
 import warnings
 
 import numpy as np
 import pytest
 
-from gpu_helpers import I, cuda, torch
+from gpu_helpers import I, O, cuda, host, torch
 
 import paper_2412_16490_gb300 as bx
 
@@ -33,7 +34,7 @@ def _launched(call, tmp_path):
 
 
 def _scene(name, B, s):
-    hand = I.hand_template(name)
+    hand = I.hand_template(name) if isinstance(name, str) else name
     obj = I.grid_object(3, n=32)
     T = I.wrench_set(12)
     T = T[:s] if s <= 12 else np.concatenate([T, np.roll(0.5 * T, 1, axis=1)[:s - 12]])
@@ -67,6 +68,93 @@ def test_several_small_jobs_take_the_wide_form(s, tmp_path):
     for tile, kernel in ((0, "multi_wide_kernel"), (8, "multi_kernel")):
         sp = bx.step_params(I.default_params(), qp=bx.qp_params(max_iter=20), grasps_per_cta=tile)
         assert _launched(lambda: bx.bodex_step_multi(jobs, sp), tmp_path) == [kernel]
+
+
+def _outputs(j, sp, steps, multi=False):
+    B = j["state"].B
+    j = dict(j, E_last=torch.empty(B, device="cuda"), status=torch.empty(B, dtype=torch.int32, device="cuda"))
+    x = j["state"].pose()
+    for n, p in zip(steps, sp if isinstance(sp, (list, tuple)) else [sp] * len(steps)):
+        if multi:
+            bx.bodex_step_multi([dict(j, n_steps=n)], p)
+        else:
+            bx.bodex_step(j["hand"], j["obj"], j["state"], j["T"], n, p, E_last=j["E_last"], status=j["status"])
+    out = [j["state"].pose(), *j["state"].adam()[:2], j["state"].residual(), j["E_last"], j["status"]]
+    j["state"].set_pose(x)
+    return out
+
+
+@pytest.mark.parametrize("name,s,B", [("hand5", 1, 40), ("hand5", 1, 2603), ("hand5", 2, 1901), ("hand5", 4, 77), ("hand4x4", 1, 1301),
+                                      ("hand4x4", 3, 1003), ("hand3", 1, 1303), ("hand3", 2, 1501)])
+@pytest.mark.parametrize("cone", [0, 1])
+@pytest.mark.parametrize("collide", [False, True])
+def test_fewer_wrenches_than_contacts_equal_the_one_lane_form(name, s, B, cone, collide, tmp_path):
+    """With s < m a step always takes the wide form, in large batches with
+    several grasps a block and as few as three lanes a grasp; the several-job
+    launch with a tile runs the same QPs a lane each."""
+    P = I.default_params(**(COLLISION if collide else {}))
+    j = _scene(name, B, s)
+    for kw in (dict(max_iter=20), dict(max_iter=60, eps_abs=1e-3, check_every=7)):
+        qp = bx.qp_params(cone=cone, **kw)
+        wide, lane = bx.step_params(P, qp=qp), bx.step_params(P, qp=qp, grasps_per_cta=8)
+        assert _launched(lambda: _step(j, wide), tmp_path) == ["fused_wide_kernel"]
+        assert _launched(lambda: bx.bodex_step_multi([dict(j, n_steps=1)], lane), tmp_path) == ["multi_kernel"]
+        j = _scene(name, B, s)
+        for a, b in zip(_outputs(j, wide, (3, 2)), _outputs(j, lane, (3, 2), multi=True)):
+            assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("name,s", [("hand3", 1), ("hand3", 2), ("hand4", 3), ("hand5", 1), ("hand5", 4)])
+@pytest.mark.parametrize("B", [33, 1777])
+def test_evaluation_with_fewer_wrenches_matches_the_oracle(name, s, B):
+    """E and dE/dx on a sphere object, every QP solved tightly (bounds as in
+    the parity tests: E relative 1e-4, gradient relative 1e-3)."""
+    hand, obj = I.hand_template(name), I.sphere_object()
+    P = I.default_params(eps_reg=1e-3)
+    x0 = I.initial_poses(hand, obj, 33, seed=7)
+    T = I.wrench_set(12)[:s]
+    sp = bx.step_params(P, qp=bx.qp_params(eps_abs=1e-6, eps_reg=1e-3, max_iter=20000, check_every=10))
+    out = bx.bodex_energy_grad(bx.Hand(hand), bx.Object(obj), cuda(np.tile(x0, (-(-B // 33), 1))[:B]), cuda(T), sp)
+    ev = O.evaluate(O.Hand(hand), O.Object(obj), x0.astype(np.float64), T, P)
+    rows = np.arange(B) % 33
+    ok = (host(out["status"]) & bx.ST_NOT_CONVERGED) == 0
+    assert ok.mean() >= 0.9
+    np.testing.assert_allclose(host(out["E"])[ok], ev["E"][rows][ok], rtol=1e-4, atol=1e-6)
+    g, ref = host(out["dEdx"]), ev["grad"][rows]
+    rel = np.linalg.norm(g - ref, axis=1) / np.maximum(np.linalg.norm(ref, axis=1), 1e-3)
+    assert (rel[ok] <= 1e-3).all(), rel[ok].max()
+
+
+@pytest.mark.parametrize("spheres", [41, 44, 48])
+@pytest.mark.parametrize("B", [5, 300])
+def test_collision_spheres_beyond_the_split_scratch(spheres, B, tmp_path):
+    """A lane per sphere needs 6 K + 9 (n + 1) words of scratch; a hand with
+    more spheres walks them by slot in the wide form too (48 spheres of the
+    22-joint hand need 495 of 490)."""
+    hand = I.hand_template("hand5")
+    more = spheres - len(hand.sphere_link)
+    pick = np.arange(more) * 5
+    hand = dataclasses.replace(hand, sphere_link=np.concatenate([hand.sphere_link, hand.sphere_link[pick]]),
+                               sphere_local=np.concatenate([hand.sphere_local, hand.sphere_local[pick] + np.float32(4e-3)]),
+                               sphere_radius=np.concatenate([hand.sphere_radius, hand.sphere_radius[pick]]))
+    P = I.default_params(**COLLISION)
+    j = _scene(hand, B, 12)
+    sp = [bx.step_params(P, qp=bx.qp_params(max_iter=20), grasps_per_cta=tile) for tile in (0, 8)]
+    assert _launched(lambda: _step(j, sp[0]), tmp_path) == ["fused_wide_kernel"]
+    j = _scene(hand, B, 12)
+    for a, b in zip(*(_outputs(j, p, (3, 2)) for p in sp)):
+        assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("name,s,B", [("hand5", 12, 100), ("hand3", 7, 64)])
+def test_a_state_moves_between_the_forms(name, s, B):
+    """The warm start of either form continues in the other."""
+    j = _scene(name, B, s)
+    wide, lane = (bx.step_params(I.default_params(), qp=bx.qp_params(max_iter=20), grasps_per_cta=t) for t in (0, 8))
+    outs = [_outputs(j, forms, (2, 3, 2)) for forms in ((lane, lane, lane), (wide, lane, wide), (lane, wide, lane))]
+    for other in outs[1:]:
+        for a, b in zip(outs[0], other):
+            assert torch.equal(a, b)
 
 
 def _times(calls, reps=9):

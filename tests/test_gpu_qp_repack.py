@@ -83,6 +83,22 @@ def test_small_batches_start_in_the_wide_form(m, cone, s, adaptive):
             assert torch.equal(large[k][first:first + 13], small[k]), (k, first)
 
 
+@pytest.mark.parametrize("m,cone", [(3, 0), (4, 0), (5, 0), (3, 1), (5, 1)])
+@pytest.mark.parametrize("s", [1, 7, 12, 16])
+@pytest.mark.parametrize("adaptive", [0, 1])
+def test_partial_last_block_of_a_large_batch(m, cone, s, adaptive):
+    """The last block's grasps, up to the batch's end, as in a small batch."""
+    T = I.wrench_set(12)
+    T = cuda(T[:s].copy() if s <= 12 else np.concatenate([T, np.roll(0.5 * T, 1, axis=1)[:s - 12]]))
+    p, n = I.random_contacts(13, m, seed=98 + m)
+    G = cuda(O.grasp_matrix(p, n).astype(np.float32))
+    prm = bx.qp_params(eps_abs=1e-5, max_iter=1500, check_every=10, adaptive_rho=adaptive, cone=cone)
+    small = bx.bodex_qp_solve_batch(G, T, prm)
+    large = bx.bodex_qp_solve_batch(G.repeat(100, 1, 1)[:1299].contiguous(), T, prm)
+    for k in ("y", "z", "lam", "Q", "iters", "status", "res"):
+        assert torch.equal(large[k][1287:1299], small[k][:12]), k
+
+
 @pytest.mark.parametrize("m", [3, 4, 5])
 @pytest.mark.parametrize("cone", [0, 1])
 def test_iterations_with_adaptive_rho_cost_as_much_as_without(m, cone):
