@@ -259,7 +259,7 @@ __global__ void __launch_bounds__(RF_THREADS) refine_kernel(RefineArgs A) {
   copy_hand_to_smem(A.hand, smem);
   const int gl = threadIdx.x / LANES, lane = threadIdx.x % LANES;
   const int b_mine = blockIdx.x * GPB + gl;
-  const int b = min(b_mine, A.B - 1);  // a group past the last grasp repeats it and writes nothing
+  const int b = WARP ? b_mine : min(b_mine, A.B - 1);  // eight lanes past the last grasp repeat it and write nothing
   const HandDev& H = *reinterpret_cast<const HandDev*>(smem);
   float* per = smem + HW + gl * PER;
   float* xs = per;
@@ -283,7 +283,6 @@ __global__ void __launch_bounds__(RF_THREADS) refine_kernel(RefineArgs A) {
   int kbest = 0;
   for (int step = 0; step < A.n_steps; ++step) {
     float* const jw = jwall + (lane < M ? lane : 0) * MAXCHAIN * 6;
-    Tf T;  // lane < M: contact lane's link frame
     if constexpr (WARP) {
       for (int e = lane; e <= H.n; e += 32) fk_joint(H, e, xs, per + oRQ, per + oRQ + 9 * MAXJ);
       __syncwarp();
@@ -293,18 +292,22 @@ __global__ void __launch_bounds__(RF_THREADS) refine_kernel(RefineArgs A) {
       __syncwarp();
 #pragma unroll
       for (int i = 0; i < M; ++i) {
+        Tf T;
         load_frame(frames + 12 * i, T);
         float phi;
         const int k = lowest_sample(T, A.tips + (size_t)i * S * 3, S, A.obj, phi);
         if (lane == i) kbest = k;
       }
-      if (lane < M) load_frame(frames + 12 * lane, T);
-    } else if (lane < M) {
-      fk_link(H, lane, xs, T, jw);
-      float phi;
-      kbest = lowest_sample_lane(T, A.tips + (size_t)lane * S * 3, S, A.obj, phi);
     }
     if (lane < M) {
+      Tf T;
+      if constexpr (WARP) {
+        load_frame(frames + 12 * lane, T);
+      } else {
+        fk_link(H, lane, xs, T, jw);
+        float phi;
+        kbest = lowest_sample_lane(T, A.tips + (size_t)lane * S * 3, S, A.obj, phi);
+      }
       const float* tip = A.tips + (size_t)lane * S * 3;
       const float sk[3] = {__ldg(tip + 3 * kbest), __ldg(tip + 3 * kbest + 1), __ldg(tip + 3 * kbest + 2)};
       float cf[3];
@@ -360,7 +363,7 @@ __global__ void __launch_bounds__(RF_THREADS) refine_kernel(RefineArgs A) {
     }
     __syncwarp();
   }
-  if (b_mine >= A.B) return;
+  if (!WARP && b_mine >= A.B) return;
   for (int k = lane; k < D; k += LANES) {
     A.x[(size_t)b * D + k] = xs[k];
     A.am[(size_t)b * D + k] = ams[k];
@@ -401,7 +404,7 @@ __global__ void __launch_bounds__(RF_THREADS) metrics_kernel(MetricsArgs A) {
   copy_hand_to_smem(A.hand, smem);
   const int gl = threadIdx.x / LANES, lane = threadIdx.x % LANES;
   const int b_mine = blockIdx.x * GPB + gl;
-  const int b = min(b_mine, A.B - 1);  // a group past the last grasp repeats it and writes nothing
+  const int b = WARP ? b_mine : min(b_mine, A.B - 1);  // eight lanes past the last grasp repeat it and write nothing
   const HandDev& H = *reinterpret_cast<const HandDev*>(smem);
   float* xs = smem + HW + gl * PER;
   float* frames = xs + align4(MAXD);  // WARP
@@ -411,32 +414,30 @@ __global__ void __launch_bounds__(RF_THREADS) metrics_kernel(MetricsArgs A) {
   for (int k = lane; k < D; k += LANES) xs[k] = A.x[(size_t)b * D + k];
   __syncwarp();
   float d = 0.f;
-  Tf T;  // lane < M: contact lane's link frame
-  if constexpr (WARP) {
+  if constexpr (WARP) {  // S > 0
     for (int e = lane; e <= H.n; e += 32) fk_joint(H, e, xs, xs + oRQ, xs + oRQ + 9 * MAXJ);
     __syncwarp();
     if (lane < 3 * M)
       fk_row(H, lane / 3, lane % 3, xs + oRQ, xs + oRQ + 9 * MAXJ, nullptr, nullptr, frames + 12 * (lane / 3), nullptr);
     __syncwarp();
-    if (S > 0) {
 #pragma unroll
-      for (int i = 0; i < M; ++i) {
-        load_frame(frames + 12 * i, T);
-        float phi;
-        (void)lowest_sample(T, A.tips + (size_t)i * S * 3, S, A.obj, phi);
-        if (lane == i) d = phi;
-      }
-    } else if (lane < M) {
-      load_frame(frames + 12 * lane, T);
+    for (int i = 0; i < M; ++i) {
+      Tf T;
+      load_frame(frames + 12 * i, T);
+      float phi;
+      (void)lowest_sample(T, A.tips + (size_t)i * S * 3, S, A.obj, phi);
+      if (lane == i) d = phi;
     }
   } else if (lane < M) {
+    Tf T;
     fk_link(H, lane, xs, T, nullptr);
-    if (S > 0) (void)lowest_sample_lane(T, A.tips + (size_t)lane * S * 3, S, A.obj, d);
-  }
-  if (S == 0 && lane < M) {
-    float c[3];
-    tf_point(T, H.clocal[lane], c);
-    d = sdf_query(A.obj, c).phi - H.alpha;
+    if (S > 0) {
+      (void)lowest_sample_lane(T, A.tips + (size_t)lane * S * 3, S, A.obj, d);
+    } else {
+      float c[3];
+      tf_point(T, H.clocal[lane], c);
+      d = sdf_query(A.obj, c).phi - H.alpha;
+    }
   }
   // spread over the grasp's fingers (in its lowest eight lanes)
   float lo = lane < M ? d : INFINITY, hi = lane < M ? d : -INFINITY;
@@ -445,7 +446,7 @@ __global__ void __launch_bounds__(RF_THREADS) metrics_kernel(MetricsArgs A) {
     lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, off));
     hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, off));
   }
-  if (b_mine >= A.B) return;
+  if (!WARP && b_mine >= A.B) return;
   if (lane < M) A.d[(size_t)b * M + lane] = d;
   if (lane == 0 && A.cdc) A.cdc[b] = hi - lo;
 }
