@@ -248,9 +248,10 @@ typedef struct bodex_step_params {
   bodex_energy_params energy;
   bodex_qp_params qp;
   int grasps_per_cta;  /* CTA tile: grasps per thread block (0 = default: 96 / s, or the
-                          form with m lanes per QP where a batch is too small to fill
-                          the GPU; the results are the same); an
-                          autotuner knob that changes speed, never results */
+                          form with m lanes per QP where that is estimated to be the
+                          faster one; the results are the same).  A requested tile
+                          runs one lane per QP (with s < m wrenches m lanes all the
+                          same).  An autotuner knob that changes speed, never results */
   int work_pulling;    /* bodex_step_multi only.  0: one thread block per tile (a job's
                           grasps_per_cta grasps), the jobs' tiles in the caller's order,
                           scheduled onto the SMs by the hardware.  1: a persistent grid of
@@ -351,9 +352,12 @@ int bodex_step_multi(const bodex_job* jobs, int n_jobs, const bodex_step_params*
 
 /* The CTA tile the fused step kernel uses for m contacts and s wrenches:
  * `requested` grasps per thread block (0: the default, 96 / s), capped by
- * 96 lanes and by the shared memory of one block.  A job of B grasps then
- * occupies ceil(B / tile) thread blocks, which is how a scheduler fills one
- * wave of the GPU (4 blocks per SM).  Host-only: touches no device.
+ * 96 lanes and by the shared memory of one block.  With one lane per QP a job
+ * of B grasps then occupies ceil(B / tile) thread blocks, which is how a
+ * scheduler fills one wave of the GPU (4 blocks per SM).  A default launch
+ * that leaves the GPU partly idle may run m lanes per QP instead, in more and
+ * other blocks: it does so only where that is the faster form, so the count
+ * stays a sound budget.  Host-only: touches no device.
  * Errors: BODEX_ERR_INVALID (m outside 3..5, s outside 1..16,
  * requested < 0, null output). */
 int bodex_step_tile(int m, int s, int requested, int* grasps_per_cta);

@@ -212,7 +212,9 @@ class Server(_Base):
             hbm_budget = int(free * 0.8)
         self.hbm_budget = int(hbm_budget)
         # thread blocks resident at once: a launch beyond one wave slows every
-        # job in it, so admission stops there (None: no limit)
+        # job in it, so admission stops there (None: no limit).  Counted in
+        # blocks of the form with a lane per QP, the one that runs when a wave
+        # is full; a launch that leaves the GPU idle may take another form
         sms = torch.cuda.get_device_properties(torch.cuda.current_device()).multi_processor_count
         self.cta_budget = None if max_waves is None else max(1, int(max_waves * sms * CTAS_PER_SM))
         self.ctas = 0
