@@ -253,7 +253,8 @@ typedef struct bodex_step_params {
                           runs one lane per QP (with s < m wrenches m lanes all the
                           same).  An autotuner knob that changes speed, never results */
   int work_pulling;    /* bodex_step_multi only.  0: one thread block per tile (a job's
-                          grasps_per_cta grasps), the jobs' tiles in the caller's order,
+                          grasps_per_cta grasps), the jobs' tiles in the caller's order
+                          (exact QPs of several contact counts: count by count),
                           scheduled onto the SMs by the hardware.  1: a persistent grid of
                           as many blocks as fit on the GPU at once; each block takes the
                           next tile from one atomic counter, the tiles of the costliest

@@ -1526,8 +1526,9 @@ struct MultiArgs {
   int total;                            // work items
   int* counter;                         // next work item (device, zeroed before the launch)
   int m[BODEX_MAX_JOBS];
-  int order_job[BODEX_MAX_JOBS];        // jobs in decreasing cost
+  int order_job[BODEX_MAX_JOBS];        // the jobs in the order of their items
   int order_begin[BODEX_MAX_JOBS + 1];  // first item of the k-th job in that order
+  int rows, cols;                       // rows > 0: of each rows * cols blocks, b, b + cols, b + 2 cols ... take consecutive items
   FusedArgs job[BODEX_MAX_JOBS];
 };
 
@@ -1575,7 +1576,15 @@ template <bool ADAPT, bool EXACT = false, bool PULL = false>
 __global__ void __launch_bounds__(CTA_LANES, 4) multi_kernel(const __grid_constant__ MultiArgs A) {
   extern __shared__ __align__(16) float smem[];
   if constexpr (!PULL) {
-    multi_item<ADAPT, EXACT>(A, (int)blockIdx.x, smem);  // one item per CTA, no loop
+    int w = (int)blockIdx.x;
+    if (EXACT && A.rows > 0) {
+      // in waves of rows x cols blocks; column c of a wave has `rows` items,
+      // or, in the last one, one fewer from column `full` on
+      const int size = A.rows * A.cols, w0 = w / size * size, n = min(size, A.total - w0), i = w - w0;
+      const int rows = (n + A.cols - 1) / A.cols, full = n - A.cols * (rows - 1), c = i % A.cols, r = i / A.cols;
+      w = w0 + (c < full ? c * rows + r : full * rows + (c - full) * (rows - 1) + r);
+    }
+    multi_item<ADAPT, EXACT>(A, w, smem);  // one item per CTA, no loop
   } else {
     __shared__ int item;
 #pragma unroll 1
@@ -1693,13 +1702,18 @@ struct FormLoad {
   int m, s, gpb, blocks, steps;
 };
 
+// Blocks of a step kernel that an SM holds at once (by registers, 16 warps of
+// the wide form or 12, and by shared memory).
+inline int resident_blocks(bool wide, int threads, size_t bytes) {
+  constexpr size_t kSmemPerSM = 228 * 1024, kReserved = 1024;  // 1 KB of every block is the system's
+  return std::max(1, std::min((wide ? 16 : 12) / ((threads + 31) / 32), (int)(kSmemPerSM / (bytes + kReserved))));
+}
+
 // Estimated time of a launch of n jobs' blocks, `threads` wide with `bytes`
 // of shared memory each, us.
 inline double form_time(bool wide, const FormLoad* job, int n, int threads, size_t bytes, const AdmmCfg& c, bool coll,
                         int sms) {
-  constexpr size_t kSmemPerSM = 228 * 1024, kReserved = 1024;  // 1 KB of every block is the system's
-  const int wpb = (threads + 31) / 32;
-  const int resident = std::max(1, std::min((wide ? 16 : 12) / wpb, (int)(kSmemPerSM / (bytes + kReserved))));
+  const int wpb = (threads + 31) / 32, resident = resident_blocks(wide, threads, bytes);
   // with a residual target the QPs of a warp rarely all stop early; beyond
   // 300 iterations the set-up no longer matters
   const double iters = c.eps > 0.f ? std::min(c.iters, 300) : c.iters;

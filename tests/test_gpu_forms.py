@@ -205,3 +205,44 @@ def test_default_form_of_several_jobs_is_not_the_slower_one(mix, s, collide):
     sp = [bx.step_params(P, qp=bx.qp_params(max_iter=20), grasps_per_cta=tile) for tile in (0, 96 // s)]
     auto, lane = _times([(reset, lambda p=p: bx.bodex_step_multi(jobs, p)) for p in sp])
     assert auto <= 1.15 * lane, (auto, lane)
+
+
+MIX = ("hand5", "hand5", "hand4x4", "hand4x4", "hand3")
+
+
+@pytest.mark.parametrize("names", [MIX, ("hand5", "hand3"), ("hand3", "hand4x4", "hand5") * 2])
+@pytest.mark.parametrize("total", [1000, 3000, 4864, 5700, 6500, 9000])
+def test_several_jobs_with_exact_qps_take_no_longer_than_their_widest_hand(names, total):
+    """Several contact counts with exact QPs in one launch: the SMs run one
+    count's code each (1.0 to 1.3 times one hand's job of as many grasps when
+    this was written; up to 2.7 times with three counts' code on every SM)."""
+    sp = bx.step_params(I.default_params(), qp=bx.qp_params(max_iter=64, solver=bx.QP_EXACT))
+    calls = []
+    for group in (names, ("hand5",)):
+        jobs = [dict(_scene(n, total // len(group), 12), n_steps=5) for n in group]
+        xs = [j["state"].pose() for j in jobs]
+
+        def reset(jobs=jobs, xs=xs):
+            for j, x in zip(jobs, xs):
+                j["state"].set_pose(x)
+
+        calls.append((reset, lambda jobs=jobs: bx.bodex_step_multi(jobs, sp)))
+    mixed, one = _times(calls, reps=5)
+    assert mixed <= 1.6 * one, (mixed, one)
+
+
+@pytest.mark.parametrize("sizes", [(40, 30, 20), (900, 700, 803), (1500, 1300, 1207), (2100, 1800, 1701), (2600, 2500, 2401)])
+@pytest.mark.parametrize("order", [("hand3", "hand5", "hand4x4"), ("hand4x4", "hand3", "hand5")])
+def test_exact_items_in_any_order_equal_the_jobs_alone(sizes, order):
+    """Up to, at and beyond the sizes whose items are laid out by SM, last
+    tiles partial: each job as in its own launch."""
+    sp = bx.step_params(I.default_params(), qp=bx.qp_params(max_iter=64, solver=bx.QP_EXACT))
+    jobs = [_scene(n, B, 12) for n, B in zip(order, sizes)]
+    alone = [_outputs(j, sp, (2,)) for j in jobs]
+    for j in jobs:
+        B = j["state"].B
+        j.update(n_steps=2, E_last=torch.empty(B, device="cuda"), status=torch.empty(B, dtype=torch.int32, device="cuda"))
+    bx.bodex_step_multi(jobs, sp)
+    for j, want in zip(jobs, alone):
+        for a, b in zip([j["state"].pose(), *j["state"].adam()[:2], j["state"].residual(), j["E_last"], j["status"]], want):
+            assert torch.equal(a, b)
