@@ -885,7 +885,7 @@ __device__ __forceinline__ void fused_cta(const FusedArgs& A, int cta, int GPB, 
     if (MODE != MODE_ADJOINT && !A.dfc && CONE != CONE_EXACT) {
       if constexpr (ADAPT) {
         AdmmCfg cg = cfg;
-        cg.rho = sc[3];
+        if (active) cg.rho = sc[3];  // a several-job block has threads beyond its job's grasps: no record there
         setup_kinv<M, true>(active, lane, S, Gs, per + L::oK, kin, cg);
       } else {
         setup_kinv<M, true>(active, lane, S, Gs, per + L::oK, kin, cfg);
@@ -965,8 +965,8 @@ __device__ __forceinline__ void fused_cta(const FusedArgs& A, int cta, int GPB, 
         float mq[NV];
         float rp = 0.f, rd = 0.f;
         AdmmCfg cg = cfg;
-        cg.rho = sc[3];
         if (active) {
+          cg.rho = sc[3];
           if (MODE == MODE_STEP) {
 #pragma unroll
             for (int a = 0; a < NV; ++a) y[a] = A.qy[a * NQ + q];

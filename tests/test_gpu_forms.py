@@ -246,3 +246,26 @@ def test_exact_items_in_any_order_equal_the_jobs_alone(sizes, order):
     for j, want in zip(jobs, alone):
         for a, b in zip([j["state"].pose(), *j["state"].adam()[:2], j["state"].residual(), j["E_last"], j["status"]], want):
             assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("cone", [0, 1])
+@pytest.mark.parametrize("few", [("hand5", 1), ("hand5", 2), ("hand3", 1), ("hand4x4", 1), ("hand4x4", 2)])
+@pytest.mark.parametrize("tile", [0, 1, 3])
+def test_adaptive_jobs_with_threads_beyond_their_grasps(few, tile, cone):
+    """Several jobs with adaptive rho in blocks of 96 threads: where shared
+    memory or a requested tile leaves a job fewer grasps a block than its
+    wrenches would, the threads beyond them have no record to read (that read
+    was out of bounds).  Each job as with full blocks, or alone."""
+    qp = bx.qp_params(max_iter=60, eps_abs=1e-3, check_every=7, adaptive_rho=1, cone=cone)
+    sizes = (("hand5", 5, 40), ("hand3", 12, 33), (*few, 165))
+    outs = []
+    for t, group in ((tile, sizes), (0, sizes[:2])):
+        sp = bx.step_params(I.default_params(), qp=qp, grasps_per_cta=t)
+        jobs = [dict(_scene(n, B, s), n_steps=3, E_last=torch.empty(B, device="cuda"),
+                     status=torch.empty(B, dtype=torch.int32, device="cuda")) for n, s, B in group]
+        bx.bodex_step_multi(jobs, sp)
+        outs.append([[j["state"].pose(), *j["state"].adam()[:2], j["state"].residual(), j["E_last"], j["status"]] for j in jobs])
+    alone = _outputs(_scene(few[0], 165, few[1]), bx.step_params(I.default_params(), qp=qp), (3,))
+    for got, want in zip(outs[0], [*outs[1], alone]):
+        for a, b in zip(got, want):
+            assert torch.equal(a, b)
