@@ -794,15 +794,17 @@ __device__ __forceinline__ void fused_cta(const FusedArgs& A, int cta, int GPB, 
   const int gl = threadIdx.x / S, lane = threadIdx.x % S;
   const int b = cta * GPB + gl;
   const bool active = (gl < GPB) && (b < A.B);
-  // With s < m lanes a grasp, a lane takes several contacts.  The kernels of
-  // one cone do without that loop, which cost the fixed-iteration step 0.8%
+  // With s < m lanes a grasp, a lane takes several contacts.  The kernels for
+  // s >= m do without that loop, which cost the fixed-iteration step 0.8%
   // (13.63 against 13.51 ms for 4096 grasps x 200 steps), the adaptive one of
   // five contacts 5% (310 -> 326 us for 3 steps of 2000 grasps) and its
   // evaluation 10% (349 -> 385 us at 810 grasps), where it spills the iterate
   // (816 bytes of loads instead of 384): run_fused gives their s < m cases to
   // the wide form or, with adaptive rho and under DFC, to the kernels for few
-  // wrenches (FEW).
-  constexpr bool ONE_CONTACT = !FEW && MODE != MODE_ADJOINT && (CONE == CONE_PYR || CONE == CONE_SOC);
+  // wrenches (FEW).  Of the several-job kernels only the adaptive one gains by
+  // it (856 bytes of loads instead of 1512; 1 to 4.5% a launch: 434 -> 417 us
+  // for 4050 grasps of hand5, 3 steps of 8 wrenches): the others are FEW.
+  constexpr bool ONE_CONTACT = !FEW && MODE != MODE_ADJOINT && CONE != CONE_EXACT;
   const HandDev& H = *reinterpret_cast<const HandDev*>(smem);
   float* kin = smem + L::HAND_WORDS + gl * L::KS;
   float* per = smem + L::HAND_WORDS + GPB * L::KS + gl * L::PER;
@@ -1535,7 +1537,7 @@ struct MultiArgs {
 static_assert(sizeof(MultiArgs) <= 32000, "job table must fit in the kernel parameter space");
 
 // Work item w: the k-th job in the item order, the tile w - order_begin[k].
-template <bool ADAPT, bool EXACT>
+template <bool ADAPT, bool EXACT, bool FEW>
 __device__ __forceinline__ void multi_item(const MultiArgs& A, int w, float* smem) {
   constexpr int CN = EXACT ? CONE_EXACT : CONE_ANY;
   int k = 0;
@@ -1544,9 +1546,9 @@ __device__ __forceinline__ void multi_item(const MultiArgs& A, int w, float* sme
   const FusedArgs& J = A.job[j];
   const int cta = w - A.order_begin[k];
   switch (A.m[j]) {
-    case 3: fused_cta<3, MODE_STEP, CN, ADAPT>(J, cta, J.gpb, smem); break;
-    case 4: fused_cta<4, MODE_STEP, CN, ADAPT>(J, cta, J.gpb, smem); break;
-    default: fused_cta<5, MODE_STEP, CN, ADAPT>(J, cta, J.gpb, smem); break;
+    case 3: fused_cta<3, MODE_STEP, CN, ADAPT, FEW>(J, cta, J.gpb, smem); break;
+    case 4: fused_cta<4, MODE_STEP, CN, ADAPT, FEW>(J, cta, J.gpb, smem); break;
+    default: fused_cta<5, MODE_STEP, CN, ADAPT, FEW>(J, cta, J.gpb, smem); break;
   }
 }
 
@@ -1572,7 +1574,8 @@ __global__ void __launch_bounds__(WIDE_THREADS, 4) multi_wide_kernel(const __gri
   }
 }
 
-template <bool ADAPT, bool EXACT = false, bool PULL = false>
+// FEW: some job may have fewer wrenches than contacts (see fused_cta).
+template <bool ADAPT, bool EXACT = false, bool PULL = false, bool FEW = true>
 __global__ void __launch_bounds__(CTA_LANES, 4) multi_kernel(const __grid_constant__ MultiArgs A) {
   extern __shared__ __align__(16) float smem[];
   if constexpr (!PULL) {
@@ -1584,7 +1587,7 @@ __global__ void __launch_bounds__(CTA_LANES, 4) multi_kernel(const __grid_consta
       const int rows = (n + A.cols - 1) / A.cols, full = n - A.cols * (rows - 1), c = i % A.cols, r = i / A.cols;
       w = w0 + (c < full ? c * rows + r : full * rows + (c - full) * (rows - 1) + r);
     }
-    multi_item<ADAPT, EXACT>(A, w, smem);  // one item per CTA, no loop
+    multi_item<ADAPT, EXACT, FEW>(A, w, smem);  // one item per CTA, no loop
   } else {
     __shared__ int item;
 #pragma unroll 1
@@ -1594,7 +1597,7 @@ __global__ void __launch_bounds__(CTA_LANES, 4) multi_kernel(const __grid_consta
       const int w = item;
       __syncthreads();  // every thread has read the item before thread 0 takes the next
       if (w >= A.total) break;
-      multi_item<ADAPT, EXACT>(A, w, smem);
+      multi_item<ADAPT, EXACT, FEW>(A, w, smem);
       __syncthreads();  // shared memory is free for the next item
     }
   }
@@ -1805,7 +1808,7 @@ inline int run_fused(int mode, const FusedArgs& A0, cudaStream_t st) {
   FusedArgs A = A0;
   const bool soc = A.cfg.cone != 0;
   const bool adapt = A.cfg.eps > 0.f && A.cfg.adapt;
-  const bool few = A.S < M;  // fewer wrenches than contacts: not in the one-lane kernels of one cone (ONE_CONTACT)
+  const bool few = A.S < M;  // fewer wrenches than contacts (ONE_CONTACT)
   // the wide form: ADMM at a fixed rho, where it pays and no tile is asked
   // for, and fewer wrenches than contacts
   bool wide = mode != MODE_ADJOINT && A.cfg.solver != BODEX_QP_EXACT && !adapt && !A.dfc;

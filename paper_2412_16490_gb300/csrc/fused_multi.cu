@@ -24,7 +24,10 @@ int launch_multi(bool adapt, bool exact, bool pull, const MultiArgs& MA, size_t 
     return adapt ? go(multi_kernel<true, false, true>) : go(multi_kernel<false, false, true>);
   }
   if (exact) return go(multi_kernel<false, true>);
-  return adapt ? go(multi_kernel<true>) : go(multi_kernel<false>);
+  if (!adapt) return go(multi_kernel<false>);
+  bool few = false;  // a job with fewer wrenches than contacts
+  for (int j = 0; j < MA.n_jobs; ++j) few |= MA.job[j].S < MA.m[j];
+  return few ? go(multi_kernel<true>) : go(multi_kernel<true, false, false, false>);
 }
 
 int launch_multi_wide(bool soc, const MultiArgs& MA, int threads, size_t bytes, cudaStream_t st) {

@@ -18,7 +18,7 @@ pytestmark = pytest.mark.gpu
 COLLISION = dict(w_pen=100.0, w_self=100.0, w_lim=10.0, eta_pen=0.005, eta_lim=0.05)
 
 
-def _launched(call, tmp_path):
+def _launched(call, tmp_path, names=r"(fused_wide_kernel|fused_kernel|multi_wide_kernel|multi_kernel)"):
     """Names of the step kernels that `call` launches."""
     call()
     torch.cuda.synchronize()
@@ -30,7 +30,7 @@ def _launched(call, tmp_path):
     with warnings.catch_warnings():
         warnings.simplefilter("ignore")  # the dump announces itself
         g.debug_dump(str(path))
-    return re.findall(r"(fused_wide_kernel|fused_kernel|multi_wide_kernel|multi_kernel)", path.read_text())
+    return re.findall(names, path.read_text())
 
 
 def _scene(name, B, s):
@@ -269,3 +269,26 @@ def test_adaptive_jobs_with_threads_beyond_their_grasps(few, tile, cone):
     for got, want in zip(outs[0], [*outs[1], alone]):
         for a, b in zip(got, want):
             assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("cone", [0, 1])
+@pytest.mark.parametrize("few", [("hand5", 4), ("hand3", 2), ("hand4x4", 1)])
+def test_adaptive_jobs_alone_and_beside_one_of_few_wrenches(few, cone, tmp_path):
+    """Several jobs with adaptive rho run in a kernel without the loop over
+    contacts, unless one has fewer wrenches than contacts; the same bits."""
+    sp = bx.step_params(I.default_params(), qp=bx.qp_params(max_iter=60, eps_abs=1e-3, check_every=7, adaptive_rho=1, cone=cone))
+    names = (("hand5", 5, 201), ("hand3", 3, 33), ("hand4x4", 12, 803), ("hand5", 12, 8))
+    kernels, outs = [], []
+    for extra in ((), ((*few, 65),)):
+        jobs = []
+        for n, s, B in names + extra:
+            jobs.append(dict(_scene(n, B, s), n_steps=3, E_last=torch.empty(B, device="cuda"),
+                             status=torch.empty(B, dtype=torch.int32, device="cuda")))
+        bx.bodex_step_multi(jobs, sp)
+        outs.append([a for j in jobs[:4] for a in (j["state"].pose(), *j["state"].adam()[:2], j["state"].residual(),
+                                                   j["E_last"], j["status"])])
+        (kernel,) = _launched(lambda: bx.bodex_step_multi(jobs, sp), tmp_path, r"multi_kernel[\w<>, ]*")
+        kernels.append(kernel)
+    for a, b in zip(*outs):
+        assert torch.equal(a, b)
+    assert kernels[0] != kernels[1]
