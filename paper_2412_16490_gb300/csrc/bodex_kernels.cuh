@@ -1729,10 +1729,13 @@ inline double form_time(bool wide, const FormLoad* job, int n, int threads, size
   const bool mixed = counts == (1 << 3 | 1 << 4 | 1 << 5);
   double t = 0;
   bool first = true;
+  long long begun = 0;  // blocks of the waves so far
   for (long long per = (total + sms - 1) / sms; per > 0; first = false) {
     const int r = (int)std::min<long long>(per, resident), warps = r * wpb, u = std::min((warps + 3) / 4, 4);
     per -= r;
     double mean = 0, longest = 0;
+    begun += (long long)r * sms;
+    long long end = 0;  // of the k-th job's blocks, which start in the order of the jobs
     for (int k = 0; k < n; ++k) {
       const FormCost& f = form_cost(wide, job[k].m);
       const double g = (double)r * job[k].gpb;
@@ -1740,9 +1743,15 @@ inline double form_time(bool wide, const FormLoad* job, int n, int threads, size
                       : f.set + f.grasp * g + f.warp * warps + f.inv_s / job[k].s;
       v = job[k].steps * (v + iters * (c.cone ? f.soc : f.pyr)[u - 1]);
       mean += v * job[k].blocks / total;
-      longest = std::max(longest, v);
+      end += job[k].blocks;
+      if (wide || end > begun - (long long)r * sms) longest = std::max(longest, v);
     }
-    double wave = per > 0 ? mean : longest;  // the launch ends with its longest blocks
+    // The launch ends with its longest blocks: in the one-lane form the
+    // longest of the last wave's jobs (three jobs of hand5 and one of hand3,
+    // 8 wrenches, cone, 4050 grasps: the last wave is hand3's alone, 272 us
+    // where the wide form takes 366); in the wide form, whose waves of small
+    // blocks drift apart with unequal step counts, the longest of all.
+    double wave = per > 0 ? mean : longest;
     // three contact counts on an SM: the wide form's many small blocks run
     // three kernels' code at once (measured against the estimates: 1.13 to
     // 1.26 with four warps a scheduler, 1.08 below, 1.06 for the cone)

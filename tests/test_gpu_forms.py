@@ -292,3 +292,21 @@ def test_adaptive_jobs_alone_and_beside_one_of_few_wrenches(few, cone, tmp_path)
     for a, b in zip(*outs):
         assert torch.equal(a, b)
     assert kernels[0] != kernels[1]
+
+
+@pytest.mark.parametrize("names,s,total,cone,iters,steps", [
+    (("hand5", "hand5", "hand5", "hand3"), 8, 4050, 1, 40, (4,)), (("hand5", "hand5", "hand5", "hand3"), 8, 4400, 1, 40, (4,)),
+    (("hand5", "hand5", "hand5", "hand3"), 12, 4700, 0, 30, (2, 8, 5)), (("hand5", "hand5", "hand5", "hand3"), 8, 3150, 0, 30, (2, 8, 5))])
+def test_unequal_jobs_do_not_take_the_slower_form(names, s, total, cone, iters, steps):
+    """The one-lane form's last wave is the cheap job's alone; the wide form's
+    waves drift apart where the jobs' steps differ."""
+    jobs = [dict(_scene(n, total // len(names), s), n_steps=steps[i % len(steps)]) for i, n in enumerate(names)]
+    xs = [j["state"].pose() for j in jobs]
+
+    def reset():
+        for j, x in zip(jobs, xs):
+            j["state"].set_pose(x)
+
+    sp = [bx.step_params(I.default_params(), qp=bx.qp_params(max_iter=iters, cone=cone), grasps_per_cta=tile) for tile in (0, 96 // s)]
+    auto, lane = _times([(reset, lambda p=p: bx.bodex_step_multi(jobs, p)) for p in sp])
+    assert auto <= 1.15 * lane, (auto, lane)
