@@ -13,7 +13,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 # translation units, compiled in parallel: the C ABI and small kernels, then
 # the heavy kernel families (see bodex_kernels.cuh)
-UNITS = ["bodex.cu", "qp.cu", "fused_m3.cu", "fused_m4.cu", "fused_m5.cu", "fused_multi.cu"]
+UNITS = ["bodex.cu", "qp.cu", "fused_m3.cu", "fused_m4.cu", "fused_m5.cu", "fused_multi.cu", "fused_multi_pull.cu"]
 SRC = [os.path.join(CSRC, u) for u in UNITS]
 DEPS = SRC + [os.path.join(CSRC, "bodex_device.cuh"), os.path.join(CSRC, "bodex_kernels.cuh"),
               os.path.join(ROOT, "include", "bodex.h")]

@@ -1206,7 +1206,9 @@ int bodex_step_multi(const bodex_job* jobs, int n_jobs, const bodex_step_params*
         return cuda_fail(e, "cudaMemsetAsync(work counter)");
       }
     }
-    r = wide ? launch_multi_wide(soc, *MA, threads, wide_bytes, st) : launch_multi(adapt, exact, pull, *MA, bytes, st);
+    r = wide   ? launch_multi_wide(soc, *MA, threads, wide_bytes, st)
+        : pull ? launch_multi_pull(adapt, exact, *MA, bytes, st)
+               : launch_multi(adapt, exact, *MA, bytes, st);
     if (r == BODEX_OK)
       for (int k = 0; k < nj; ++k) jobs[take[k]].state->t += jobs[take[k]].n_steps;
   }

@@ -1,9 +1,9 @@
 // Kernels and launch helpers shared by the library's translation units:
 // the per-grasp shared-memory layout, the batched-QP kernel, the fused
 // step kernel and the several-job kernel.  bodex.cu holds the C ABI and the
-// small kernels; qp.cu, fused_m3.cu, fused_m4.cu, fused_m5.cu and
-// fused_multi.cu instantiate the heavy kernels, so that nvcc compiles them
-// in parallel.
+// small kernels; qp.cu, fused_m3.cu, fused_m4.cu, fused_m5.cu,
+// fused_multi.cu and fused_multi_pull.cu instantiate the heavy kernels, so
+// that nvcc compiles them in parallel.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -801,9 +801,11 @@ __device__ __forceinline__ void fused_cta(const FusedArgs& A, int cta, int GPB, 
   // evaluation 10% (349 -> 385 us at 810 grasps), where it spills the iterate
   // (816 bytes of loads instead of 384): run_fused gives their s < m cases to
   // the wide form or, with adaptive rho and under DFC, to the kernels for few
-  // wrenches (FEW).  Of the several-job kernels only the adaptive one gains by
-  // it (856 bytes of loads instead of 1512; 1 to 4.5% a launch: 434 -> 417 us
-  // for 4050 grasps of hand5, 3 steps of 8 wrenches): the others are FEW.
+  // wrenches (FEW).  Launches of several jobs take the kernels for few wrenches
+  // when a job needs them (without the loop the adaptive one reloads 856 bytes
+  // instead of 1512, 434 -> 417 us for 4050 grasps of hand5, 3 steps of 8
+  // wrenches; fixed rho gains some 1%) and when blocks pull their items, whose
+  // spills without it are no smaller (8704 grasps of hand5: 637 us, with it 614).
   constexpr bool ONE_CONTACT = !FEW && MODE != MODE_ADJOINT && CONE != CONE_EXACT;
   const HandDev& H = *reinterpret_cast<const HandDev*>(smem);
   float* kin = smem + L::HAND_WORDS + gl * L::KS;
@@ -1536,6 +1538,13 @@ struct MultiArgs {
 
 static_assert(sizeof(MultiArgs) <= 32000, "job table must fit in the kernel parameter space");
 
+// Some job has fewer wrenches than contacts.
+inline bool few_wrenches(const MultiArgs& A) {
+  for (int j = 0; j < A.n_jobs; ++j)
+    if (A.job[j].S < A.m[j]) return true;
+  return false;
+}
+
 // Work item w: the k-th job in the item order, the tile w - order_begin[k].
 template <bool ADAPT, bool EXACT, bool FEW>
 __device__ __forceinline__ void multi_item(const MultiArgs& A, int w, float* smem) {
@@ -1896,7 +1905,7 @@ inline int run_qp(const float* G, int B, const float* T, int s, const AdmmCfg& c
   }
 }
 
-// Launchers, one translation unit each (fused_m*.cu, qp.cu, fused_multi.cu).
+// Launchers, one translation unit each (fused_m*.cu, qp.cu, fused_multi*.cu).
 int launch_fused_m3(int mode, const FusedArgs& A, cudaStream_t st);
 int launch_fused_m4(int mode, const FusedArgs& A, cudaStream_t st);
 int launch_fused_m5(int mode, const FusedArgs& A, cudaStream_t st);
@@ -1905,5 +1914,6 @@ int load_steps_m4();
 int load_steps_m5();
 int launch_qp(int m, const float* G, int B, const float* T, int s, const AdmmCfg& cfg, int warm, float* y, float* z,
               float* lam, float* Q, int32_t* iters, int32_t* status, float* res, cudaStream_t st);
-int launch_multi(bool adapt, bool exact, bool pull, const MultiArgs& MA, size_t bytes, cudaStream_t st);
+int launch_multi(bool adapt, bool exact, const MultiArgs& MA, size_t bytes, cudaStream_t st);
+int launch_multi_pull(bool adapt, bool exact, const MultiArgs& MA, size_t bytes, cudaStream_t st);
 int launch_multi_wide(bool soc, const MultiArgs& MA, int threads, size_t bytes, cudaStream_t st);

@@ -273,10 +273,12 @@ def test_adaptive_jobs_with_threads_beyond_their_grasps(few, tile, cone):
 
 @pytest.mark.parametrize("cone", [0, 1])
 @pytest.mark.parametrize("few", [("hand5", 4), ("hand3", 2), ("hand4x4", 1)])
-def test_adaptive_jobs_alone_and_beside_one_of_few_wrenches(few, cone, tmp_path):
-    """Several jobs with adaptive rho run in a kernel without the loop over
-    contacts, unless one has fewer wrenches than contacts; the same bits."""
-    sp = bx.step_params(I.default_params(), qp=bx.qp_params(max_iter=60, eps_abs=1e-3, check_every=7, adaptive_rho=1, cone=cone))
+@pytest.mark.parametrize("adapt", [0, 1])
+def test_jobs_alone_and_beside_one_of_few_wrenches(few, cone, adapt, tmp_path):
+    """Several jobs run in a kernel without the loop over contacts, unless one
+    has fewer wrenches than contacts; the same bits."""
+    sp = bx.step_params(I.default_params(), grasps_per_cta=8,
+                        qp=bx.qp_params(max_iter=60, eps_abs=1e-3, check_every=7, adaptive_rho=adapt, cone=cone))
     names = (("hand5", 5, 201), ("hand3", 3, 33), ("hand4x4", 12, 803), ("hand5", 12, 8))
     kernels, outs = [], []
     for extra in ((), ((*few, 65),)):
