@@ -496,23 +496,25 @@ namespace {
 // samples a finger that grows with the grasps an SM holds (g) until the batch
 // fills the GPU.  Measured at 64 to 65,536 grasps and 1 to 128 samples, us a
 // step, eight lanes -> a warp.  64^3 grid, five fingers: 2000 grasps, 2
-// samples 5.9 -> 7.6, 4: 7.6 -> 7.7, 8: 11.1 -> 7.9; 6000 grasps, 8: 14.6 ->
-// 18.9, 12: 19.2 -> 19.3, 16: 24.1 -> 19.9; 65,536 grasps, 12: 136 -> 165,
-// 16: 194 -> 170 (three fingers 16: 83 -> 107, 24: 115 -> 113; the metrics
-// cross at some 20 for every hand, hence `most`).  Sphere, whose queries are
+// samples 5.9 -> 7.6, 4: 7.6 -> 7.7, 8: 11.1 -> 7.9; 5000 grasps, 10: 16.5 ->
+// 17.9 (four fingers 13.9 -> 15.7); 6000 grasps, 8: 14.6 -> 18.9, 12: 19.2 ->
+// 19.3, 16: 24.1 -> 19.9; 65,536 grasps, 12: 136 -> 165, 16: 194 -> 170 (three
+// fingers 16: 83 -> 107, 24: 115 -> 113, and 20,000 grasps with 20 44 -> 35; the
+// metrics cross at some 18 for every hand, 28,000 grasps of three fingers with
+// 20 take 56 -> 44 us; hence `most`).  Sphere, whose queries are
 // arithmetic alone: 2000 grasps, 12: 4.3 -> 4.4, 24: 5.3 -> 4.3; 6000, 32: 8.0
 // -> 9.9, 48: 9.5 -> 11.4, 64: 11.6 -> 11.3; 65,536, 64: 76 -> 102, 128: 128
 // -> 127.  More than 32 samples are two and more rounds of the warp.
 template <int M>
 bool warp_per_grasp(const ObjDev& obj, int S, int B, double most) {
   const double g = (double)B / sm_count(), rounds = S > 32 ? 0.8 * S : S;
-  return rounds > (obj.kind == 0 ? std::min(std::max(1.0, g), 80.0) : std::min(std::max(2.0, 0.27 * g), most));
+  return rounds > (obj.kind == 0 ? std::min(std::max(1.0, g), 80.0) : std::min(std::max(2.0, 0.31 * g), most));
 }
 
 template <int M>
 int run_refine(const RefineArgs& A, cudaStream_t st) {
   (void)cudaGetLastError();
-  if (warp_per_grasp<M>(A.obj, A.S, A.B, 64.0 / M))
+  if (warp_per_grasp<M>(A.obj, A.S, A.B, std::min(19.0, 64.0 / M)))
     refine_kernel<M, 32><<<(A.B + RF_THREADS / 32 - 1) / (RF_THREADS / 32), RF_THREADS, 0, st>>>(A);
   else
     refine_kernel<M, 8><<<(A.B + RF_THREADS / 8 - 1) / (RF_THREADS / 8), RF_THREADS, 0, st>>>(A);
@@ -522,7 +524,7 @@ int run_refine(const RefineArgs& A, cudaStream_t st) {
 template <int M>
 int run_metrics(const MetricsArgs& A, cudaStream_t st) {
   (void)cudaGetLastError();
-  if (warp_per_grasp<M>(A.obj, A.S, A.B, 20.0))
+  if (warp_per_grasp<M>(A.obj, A.S, A.B, 19.0))
     metrics_kernel<M, 32><<<(A.B + RF_THREADS / 32 - 1) / (RF_THREADS / 32), RF_THREADS, 0, st>>>(A);
   else
     metrics_kernel<M, 8><<<(A.B + RF_THREADS / 8 - 1) / (RF_THREADS / 8), RF_THREADS, 0, st>>>(A);

@@ -2,6 +2,8 @@
 per grasp, by the samples, the batch and the object.  Both forms find the
 sample with the smallest phi, lowest index on ties, at any sample count."""
 import dataclasses
+import re
+import warnings
 
 import numpy as np
 import pytest
@@ -104,3 +106,28 @@ def test_few_samples_cost_less_than_many():
                 best = min(best, a.elapsed_time(b))
         ms.append(best)
     assert ms[0] <= 0.6 * ms[1], ms
+
+
+@pytest.mark.parametrize("metrics,name,S,B,lanes", [(False, "hand4", 10, 5000, 8), (False, "hand5", 10, 5000, 8), (False, "hand5", 10, 3500, 32),
+                                                    (False, "hand3", 20, 10000, 32), (False, "hand3", 20, 20000, 32),
+                                                    (True, "hand3", 20, 28000, 32), (True, "hand4", 20, 14000, 32), (True, "hand5", 10, 28000, 8)])
+def test_the_faster_form_near_the_crossings(metrics, name, S, B, lanes, tmp_path):
+    """Lanes a grasp of the launched kernel where one form was 5 to 30% faster."""
+    hand, obj, x0 = _case(name, "grid", S)
+    H, Ob = bx.Hand(hand), bx.Object(obj)
+    x = cuda(np.tile(x0, (-(-B // len(x0)), 1))[:B])
+    pc = bx.bodex_fk_contacts(H, Ob, x)["p"]
+    st, sp = bx.State(H, B, 1), bx.step_params(I.default_params())
+    st.set_pose(x)
+    call = (lambda: bx.bodex_contact_metrics(H, Ob, x)) if metrics else (lambda: bx.bodex_refine(H, Ob, st, pc, 1, 0.01, 300.0, sp))
+    call()
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph(keep_graph=True)
+    g.enable_debug_mode()
+    with torch.cuda.graph(g):
+        call()
+    with warnings.catch_warnings():
+        warnings.simplefilter("ignore")  # the dump announces itself
+        g.debug_dump(str(tmp_path / "graph.dot"))
+    launched = re.findall(r"(?:refine|metrics)_kernel(?:I|<)(?:Li)?\d(?:E|, *)(?:Li)?(\d+)", (tmp_path / "graph.dot").read_text())
+    assert launched == [str(lanes)]
